@@ -256,6 +256,12 @@ qtc_status qtc_plan_create(const qtc_network* n, const qtc_plan_opts* opts,
  * the projector networks of one circuit, Section 3.3's sequence of
  * contractions reusing one ordering).  QTC_ERR_INVALID otherwise. */
 qtc_status qtc_plan_reuse(const qtc_plan* like, const qtc_network* n, qtc_plan** out);
+/* The plan whose contraction tree the graph executor runs for p's network in
+ * element type dtype: complex128 networks with tensors above rank 10 are
+ * contracted along a tree rearranged under a model of the device's step times
+ * (fewer multiply-adds and passes over the large tensors; the same scalar),
+ * other plans come back unchanged.  Host only. */
+qtc_status qtc_plan_execution_tree(const qtc_plan* p, int dtype, qtc_plan** out);
 qtc_status qtc_plan_stats(const qtc_plan* p, qtc_plan_info* info);
 /* Writes the contraction tree: for step s, operands (lhs[s], rhs[s]) are
  * tensor ids (0..n_tensors-1 leaves, n_tensors+t the result of step t).
@@ -285,6 +291,9 @@ qtc_status qtc_batch_create(const qtc_circuit* c, const int32_t* obs_edges,
                             int m, int lightcone, int diag_mode,
                             const qtc_plan_opts* opts, qtc_batch** out);
 qtc_status qtc_batch_stats(const qtc_batch* b, qtc_batch_info* info);
+/* b's networks with the trees of qtc_plan_execution_tree: its stats are the
+ * multiply-adds and bytes that the graph executor runs for b. */
+qtc_status qtc_batch_execution_trees(const qtc_batch* b, int dtype, qtc_batch** out);
 void qtc_batch_destroy(qtc_batch* b);
 
 /* Edge networks are independent (the objective of Section 4.1 is a sum over
@@ -306,7 +315,8 @@ qtc_status qtc_batch_partition(const qtc_batch* b, int n_parts, int want_grad,
 qtc_status qtc_batch_subset(const qtc_batch* b, const int32_t* nets, int k, qtc_batch** out);
 
 /* Builds, validates and describes the batch's device program on the host
- * only (no GPU call): every access range, counter and dependency order of a
+ * only (no GPU call), along the plans' own contraction trees (an engine's graph
+ * executor runs those of qtc_batch_execution_trees): every access range, counter and dependency order of a
  * graph program is checked against its buffers.  force_graph, small_rank and
  * max_wave_bytes as in qtc_engine_set_graph_options / qtc_engine_set_limits;
  * smem_limit: shared memory per CTA to plan for (0: 227 KiB). */

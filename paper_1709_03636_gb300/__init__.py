@@ -243,6 +243,15 @@ class Plan(_Handle):
         super().__init__(h)
         self.n_params = network.n_params
 
+    def execution_tree(self, dtype="c64") -> "Plan":
+        """The plan whose tree the graph executor contracts (qtc_plan_execution_tree)."""
+        h = ctypes.c_void_p()
+        check(lib.qtc_plan_execution_tree(self.ptr, _dtype(dtype), ctypes.byref(h)))
+        plan = Plan.__new__(Plan)
+        _Handle.__init__(plan, h)
+        plan.n_params = self.n_params
+        return plan
+
     def stats(self) -> dict:
         info = qtc_plan_info()
         check(lib.qtc_plan_stats(self.ptr, ctypes.byref(info)))
@@ -329,6 +338,18 @@ class Batch(_Handle):
         sub.p = self.p
         sub.n_params = self.n_params
         return sub
+
+    def execution_trees(self, dtype="c64") -> "Batch":
+        """The same networks with the trees the graph executor contracts
+        (qtc_batch_execution_trees), e.g. for the work it really does."""
+        h = ctypes.c_void_p()
+        check(lib.qtc_batch_execution_trees(self.ptr, _dtype(dtype), ctypes.byref(h)))
+        other = Batch.__new__(Batch)
+        _Handle.__init__(other, h)
+        other.edges = list(self.edges)
+        other.p = self.p
+        other.n_params = self.n_params
+        return other
 
     def prepare(self, engine: Engine, dtype="c64", want_grad=False, stream=None):
         check(lib.qtc_batch_prepare(engine.ptr, self.ptr, _dtype(dtype), int(want_grad),

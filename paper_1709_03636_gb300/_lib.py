@@ -71,6 +71,8 @@ SIGNATURES = {
     "qtc_network_leaf_values": (c_int, [c_void_p, c_int, P(c_double), P(c_double), P(c_double)]),
     "qtc_network_destroy": (None, [c_void_p]),
     "qtc_plan_create": (c_int, [c_void_p, P(qtc_plan_opts), P(c_void_p)]),
+    "qtc_plan_execution_tree": (c_int, [c_void_p, c_int, P(c_void_p)]),
+    "qtc_batch_execution_trees": (c_int, [c_void_p, c_int, P(c_void_p)]),
     "qtc_plan_stats": (c_int, [c_void_p, P(qtc_plan_info)]),
     "qtc_plan_steps": (c_int, [c_void_p, P(c_int32), P(c_int32)]),
     "qtc_plan_step_shapes": (c_int, [c_void_p, P(c_int32)]),

@@ -196,6 +196,7 @@ extern "C" qtc_status qtc_engine_create(int device, void* arena, size_t arena_by
     cuda_check(cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device), "SM count");
     e->sm_count = v;
     e->options.sm_count = v;
+    e->options.plan_trees = false;
     cuda_check(cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, device),
                "shared memory limit");
     e->smem_optin = (size_t)v;
@@ -560,6 +561,17 @@ extern "C" qtc_status qtc_plan_reuse(const qtc_plan* like, const qtc_network* n,
   });
 }
 
+extern "C" qtc_status qtc_plan_execution_tree(const qtc_plan* p, int dtype, qtc_plan** out) {
+  return guarded([&] {
+    if (!p || !out) fail(QTC_ERR_INVALID, "null argument");
+    if (dtype != QTC_C128 && dtype != QTC_C64 && dtype != QTC_SPLIT_BF16)
+      fail(QTC_ERR_INVALID, "unknown dtype %d", dtype);
+    auto q = std::make_unique<qtc_plan>();
+    q->plan = execution_plan(p->plan, tree_model(dtype));
+    *out = q.release();
+  });
+}
+
 extern "C" qtc_status qtc_plan_stats(const qtc_plan* p, qtc_plan_info* info) {
   return guarded([&] {
     if (!p || !info) fail(QTC_ERR_INVALID, "null argument");
@@ -761,6 +773,21 @@ extern "C" qtc_status qtc_batch_subset(const qtc_batch* b, const int32_t* nets, 
       s->obs_edges.push_back(b->obs_edges[i]);
       s->weights.push_back(b->weights[i]);
     }
+    *out = s.release();
+  });
+}
+
+extern "C" qtc_status qtc_batch_execution_trees(const qtc_batch* b, int dtype, qtc_batch** out) {
+  return guarded([&] {
+    if (!b || !out) fail(QTC_ERR_INVALID, "null argument");
+    if (dtype != QTC_C128 && dtype != QTC_C64 && dtype != QTC_SPLIT_BF16)
+      fail(QTC_ERR_INVALID, "unknown dtype %d", dtype);
+    auto s = std::make_unique<qtc_batch>();
+    s->circuit = b->circuit;
+    s->qaoa_reduce = b->qaoa_reduce;
+    s->obs_edges = b->obs_edges;
+    s->weights = b->weights;
+    for (const Plan& p : b->plans) s->plans.push_back(execution_plan(p, tree_model(dtype)));
     *out = s.release();
   });
 }
@@ -1112,10 +1139,23 @@ static Prepared& prepare(qtc_engine* e, qtc_batch* b, int dtype, int want_grad,
       return p;
   const size_t max_dyn = max_dynamic_smem(e->smem_optin);
   const HostProgram& hp = host_program(b, dtype, want_grad, max_dyn, e->options);
+  if (hp.graph) {
+    const size_t used = e->used, work = e->work;
+    try {
+      return prepare_graph(e, b, hp, stream, max_dyn);
+    } catch (const Error& err) {
+      // an arena sized for the plans' own trees: contract those
+      if (err.status != QTC_ERR_ARENA) throw;
+      e->used = used;
+      e->work = work;
+    }
+    ProgramOptions own = e->options;
+    own.plan_trees = true;
+    return prepare_graph(e, b, host_program(b, dtype, want_grad, max_dyn, own), stream, max_dyn);
+  }
   const int P = hp.n_params;
   const int N = hp.n_nets;
   const int G = (int)hp.gates.size();
-  if (hp.graph) return prepare_graph(e, b, hp, stream, max_dyn);
 
   DeviceScope scope(e->device);
   Prepared pr;

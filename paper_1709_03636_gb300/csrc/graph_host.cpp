@@ -1,7 +1,10 @@
 // Host side of the graph executor: per-network units -> waves of tasks.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <queue>
+#include <system_error>
+#include <thread>
 #include <tuple>
 
 #include "qtc_internal.h"
@@ -436,8 +439,53 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
   if (lim.tensor_cores) lim.tile_mode = 0;   // the tensor-core build has no tile tasks
   // with tensor cores four teams share one CTA's shared memory
   if (lim.tensor_cores) lim.arena_elems = (uint32_t)(32768 / elem);
+  const uint64_t cap_elems = wave_cap_bytes / elem;
+  auto over = [&](const NetGraph& g) {
+    return ((g.global_elems + 63) & ~uint64_t(63)) > cap_elems;
+  };
+  // one network's units, contracting `plan`'s tree
+  auto lower_network = [&](int i, const Plan& plan) {
+    // a subtree that does not fit its arena is cut into smaller ones
+    GraphLimits li = lim;
+    NetGraph best;
+    for (;;) {
+      best = lower_graph(plan, leaf_gate[i], val_off, der_off, hp.table_elems, hp.want_grad != 0,
+                         li);
+      if (best.fits || li.subtree_elems <= 64) break;
+      li.subtree_elems /= 2;
+    }
+    if (!best.fits) return best;
+    // a network whose stored values exceed the wave limit on their own:
+    // checkpoint segments, recomputed by the adjoint sweep (fewest that fit)
+    if (over(best)) {
+      // reuse memory also where that adds write-after-read dependencies
+      GraphLimits ld = li;
+      ld.reuse_with_deps = true;
+      NetGraph g = lower_graph(plan, leaf_gate[i], val_off, der_off, hp.table_elems,
+                               hp.want_grad != 0, ld);
+      if (g.fits && g.global_elems < best.global_elems) {
+        best = std::move(g);
+        li = ld;
+      }
+    }
+    if (hp.want_grad && over(best)) {
+      for (int k : {2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64}) {
+        GraphLimits lk = li;
+        lk.reuse_with_deps = true;
+        lk.checkpoint_segments = k;
+        NetGraph g = lower_graph(plan, leaf_gate[i], val_off, der_off, hp.table_elems, true, lk);
+        if (!g.fits) break;
+        const bool ok = !over(g);
+        if (ok || g.global_elems < best.global_elems) best = std::move(g);
+        if (ok) break;
+      }
+    }
+    return best;
+  };
+  const TreeModel model = tree_model(hp.dtype);
   std::vector<NetGraph> graphs(N);
-  for (int i = 0; i < N; ++i) {
+  std::vector<Error> errors(N, Error{QTC_OK, ""});
+  auto lower_one = [&](int i) {
     // a network that fits whole in shared memory stays one fused task
     LoweredNet ln = lower_smem(plans[i], leaf_gate[i], val_off, der_off, hp.table_elems,
                                hp.want_grad != 0, hp.table_elems + lim.arena_elems);
@@ -447,57 +495,54 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
       u.ops = std::move(ln.ops);
       u.arena_elems = ln.arena_elems;
       graphs[i].units.push_back(std::move(u));
-      continue;
+      return;
     }
-    // a subtree that does not fit its arena is cut into smaller ones
-    GraphLimits li = lim;
-    for (;;) {
-      graphs[i] = lower_graph(plans[i], leaf_gate[i], val_off, der_off, hp.table_elems,
-                              hp.want_grad != 0, li);
-      if (graphs[i].fits || li.subtree_elems <= 64) break;
-      li.subtree_elems /= 2;
+    NetGraph g;
+    g.fits = false;
+    if (!opts.plan_trees) g = lower_network(i, execution_plan(plans[i], model));
+    if (!g.fits || over(g)) {
+      // the plan's own tree, where the rearranged one cannot be lowered or
+      // needs more memory than a wave may take
+      NetGraph own = lower_network(i, plans[i]);
+      if (!g.fits || (own.fits && !over(own))) g = std::move(own);
     }
-    if (!graphs[i].fits)
+    if (!g.fits)
       fail(QTC_ERR_UNSUPPORTED, "network %d (max rank %d): %s", i, plans[i].max_rank,
-           graphs[i].why.c_str());
-    // a network whose stored values exceed the wave limit on their own:
-    // checkpoint segments, recomputed by the adjoint sweep (fewest that fit)
-    const uint64_t cap_elems = wave_cap_bytes / elem;
-    auto over = [&](const NetGraph& g) {
-      return ((g.global_elems + 63) & ~uint64_t(63)) > cap_elems;
+           g.why.c_str());
+    check_global_placement(g);
+    graphs[i] = std::move(g);
+  };
+  {
+    const unsigned hw = std::max(1u, std::min({32u, std::thread::hardware_concurrency(),
+                                               (unsigned)N}));
+    std::atomic<int> next{0};
+    auto work = [&] {
+      for (int i = next++; i < N; i = next++) try {
+          lower_one(i);
+        } catch (const Error& e) {
+          errors[i] = e;
+        } catch (const std::exception& e) {
+          errors[i] = Error{QTC_ERR_INVALID, e.what()};
+        }
     };
-    if (over(graphs[i])) {
-      // reuse memory also where that adds write-after-read dependencies
-      GraphLimits ld = li;
-      ld.reuse_with_deps = true;
-      NetGraph g = lower_graph(plans[i], leaf_gate[i], val_off, der_off, hp.table_elems,
-                               hp.want_grad != 0, ld);
-      if (g.fits && g.global_elems < graphs[i].global_elems) {
-        graphs[i] = std::move(g);
-        li = ld;
-      }
+    std::vector<std::thread> pool;
+    try {
+      for (unsigned t = 1; t < hw; ++t) pool.emplace_back(work);
+    } catch (const std::system_error&) {
+      // fewer threads than asked for: the ones there are do the work
     }
-    if (hp.want_grad && over(graphs[i])) {
-      for (int k : {2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64}) {
-        GraphLimits lk = li;
-        lk.reuse_with_deps = true;
-        lk.checkpoint_segments = k;
-        NetGraph g = lower_graph(plans[i], leaf_gate[i], val_off, der_off, hp.table_elems,
-                                 true, lk);
-        if (!g.fits) break;
-        const bool ok = ((g.global_elems + 63) & ~uint64_t(63)) <= cap_elems;
-        if (ok || g.global_elems < graphs[i].global_elems) graphs[i] = std::move(g);
-        if (ok) break;
-      }
-    }
-    check_global_placement(graphs[i]);
-    hp.max_checkpoint_segments = std::max(hp.max_checkpoint_segments,
-                                          graphs[i].checkpoint_segments);
-    hp.sum_global_elems += graphs[i].global_elems;
-    hp.sum_unshared_elems += graphs[i].unshared_elems;
+    work();
+    for (auto& th : pool) th.join();
+  }
+  for (const Error& e : errors)
+    if (e.status != QTC_OK) throw e;
+  for (const NetGraph& g : graphs) {
+    hp.max_checkpoint_segments = std::max(hp.max_checkpoint_segments, g.checkpoint_segments);
+    hp.sum_global_elems += g.global_elems;
+    hp.sum_unshared_elems += g.unshared_elems;
   }
   // waves: largest networks first, first fit under the cap
-  const uint64_t cap = wave_cap_bytes / elem;
+  const uint64_t cap = cap_elems;
   std::vector<int> order(N);
   for (int i = 0; i < N; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) {

@@ -136,6 +136,21 @@ struct Plan {
 };
 
 Plan make_plan(const Network& net, const qtc_plan_opts& opts);
+// Storage order of every tensor's labels and the plan's costs, from its steps.
+void layout_labels(Plan& plan);
+
+// What a step costs on the device, for choosing the tree to execute.
+struct TreeModel {
+  double elem = 8;             // bytes per element
+  double bytes_per_ns = 6000;  // memory, all SMs
+  double macs_per_ns = 3000;   // complex multiply-adds, all SMs
+  double step_ns = 1;          // per step, over the networks that run beside it
+  int small_rank = 10;         // trees of tensors up to this rank stay as they are
+};
+// The model of an element type (qtc_dtype).
+TreeModel tree_model(int dtype);
+// The plan with a tree rearranged for execution (same network, same scalar).
+Plan execution_plan(const Plan& plan, const TreeModel& model);
 
 // ---- leaf tensors as coefficients (gate_coef.cpp) ---------------------------
 // A, B, C (2^rank each) with element = A cos(t/2) + B sin(t/2) + C.
@@ -274,12 +289,15 @@ struct ProgramOptions {
                                    // 2: per warp, steps always streamed
   int sm_count = 152;              // SMs of the device the program is laid out for
   bool graph_hi_occupancy = false; // graph executor: the five-CTAs-per-SM instantiation
+  bool plan_trees = true;          // graph executor: contract the plans' own trees; false
+                                   // (what engines run): execution_plan's
   bool operator==(const ProgramOptions& o) const {
     return wave_cap_bytes == o.wave_cap_bytes && force_graph == o.force_graph &&
            small_rank == o.small_rank && task_terms_log2 == o.task_terms_log2 &&
            tile_mode == o.tile_mode &&
            subtree_bytes == o.subtree_bytes && warp_teams == o.warp_teams &&
-           sm_count == o.sm_count && graph_hi_occupancy == o.graph_hi_occupancy;
+           sm_count == o.sm_count && graph_hi_occupancy == o.graph_hi_occupancy &&
+           plan_trees == o.plan_trees;
   }
 };
 
