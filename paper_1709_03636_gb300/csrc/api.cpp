@@ -1033,6 +1033,19 @@ const HostProgram& qtc::host_program(qtc_batch* b, int dtype, int want_grad,
   if (!ok)
     fail(QTC_ERR_UNSUPPORTED, "program needs %zu bytes of shared memory (limit %zu)", hp->smem,
          max_dynamic);
+  if (!hp->warp_teams) {
+    std::vector<SOp> all;
+    for (TaskDev& t : hp->tasks) {
+      std::vector<SOp> ops(hp->ops.begin() + t.op_begin,
+                           hp->ops.begin() + t.op_begin + t.op_count);
+      schedule_cta_ops(ops, table_elems, hp->block / 32);
+      validate_cta_ops(ops.data(), ops.size(), table_elems, hp->max_arena, 0, P, hp->block / 32);
+      t.op_begin = (uint32_t)all.size();
+      t.op_count = (uint32_t)ops.size();
+      all.insert(all.end(), ops.begin(), ops.end());
+    }
+    hp->ops = std::move(all);
+  }
   b->host_programs.push_back(std::move(hp));
   return *b->host_programs.back();
 }

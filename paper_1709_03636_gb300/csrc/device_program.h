@@ -95,11 +95,24 @@ enum SOpCode : uint8_t {
 // Operand locations: by default an op offset is an element offset into the
 // task's shared memory (gate table first, then the arena); a flagged operand
 // is an element offset into the global work buffer (graph executor only).
+//
+// A task's ops run level by level (cta_program.cpp): the ops of one level touch
+// no memory that another of them writes, and the team meets at a barrier after
+// the last of them only.  A narrow op (few outputs) is run by one warp, the
+// others of the level's narrow ops by other warps at the same time; any other
+// op by the whole team.
 enum SOpFlag : uint8_t {
   SOPF_OUT_GLOBAL = 1,
   SOPF_IN1_GLOBAL = 2,
-  SOPF_IN2_GLOBAL = 4
+  SOPF_IN2_GLOBAL = 4,
+  SOPF_NARROW = 8,     // run by warp `code >> 4` of the team
+  SOPF_SYNC = 16,      // last op of its level: team barrier after it
+  SOPF_LANES = 32,     // narrow adjoint op: the warp's lanes share each output's sum
+  SOPF_LEAFDOT = 64    // narrow adjoint of a leaf: the output is not stored; its dot with
+                       // table[out ..] (d(leaf)/dparam) is added to slot p1[kLeafSlotByte]
 };
+constexpr int kLeafSlotByte = 15;     // (a leaf's output has at most 4 bits)
+constexpr uint32_t kNarrowMax = 128;  // outputs of a narrow op
 
 constexpr int kMaxSmemRank = 16;
 constexpr uint8_t kAbsent = 0xFF;
@@ -110,7 +123,7 @@ constexpr uint8_t kAbsent = 0xFF;
 // operand does not carry that label); summed bit j reads in1 bit y1[j] and
 // in2 bit y2[j].
 struct alignas(16) SOp {
-  uint8_t code, rc, ry, flags;
+  uint8_t code, rc, ry, flags;  // code: low 4 bits SOpCode, high 4 bits the warp of a narrow op
   uint32_t out, in1, in2;
   uint8_t p1[kMaxSmemRank], p2[kMaxSmemRank];
   uint8_t y1[kMaxSmemRank], y2[kMaxSmemRank];

@@ -324,32 +324,227 @@ __device__ __forceinline__ T* resolve(uint32_t off, T* table, T* arena, uint32_t
   return off < table_elems ? table + off : arena + (off - table_elems);
 }
 
-// out = sum over the summed bits of a * b for every output element; the
-// team's threads (team.tid of team.size) share the outputs.
-template <typename T, typename TeamT>
-__device__ __forceinline__ void contract_op(const SOp& op, T* out, const T* a, const T* b,
-                                            const TeamT& team) {
-  const uint32_t nout = 1u << op.rc;
-  const uint32_t ny = 1u << op.ry;
-  for (uint32_t c = team.tid; c < nout; c += team.size) {
-    uint32_t oa = 0, ob = 0;
-    for (int i = 0; i < op.rc; ++i) {
-      const uint32_t bit = (c >> i) & 1u;
-      if (op.p1[i] != kAbsent) oa |= bit << op.p1[i];
-      if (op.p2[i] != kAbsent) ob |= bit << op.p2[i];
-    }
-    T acc = czero<T>();
-    for (uint32_t y = 0; y < ny; ++y) {
-      uint32_t ya = 0, yb = 0;
-      for (int j = 0; j < op.ry; ++j) {
-        const uint32_t bit = (y >> j) & 1u;
-        if (op.y1[j] != kAbsent) ya |= bit << op.y1[j];
-        if (op.y2[j] != kAbsent) yb |= bit << op.y2[j];
-      }
-      acc = cfma(a[oa | ya], b[ob | yb], acc);
-    }
-    out[c] = acc;
+// v << n, zero for n >= 32 (PTX clamps; an absent label's position is 255).
+__device__ __forceinline__ uint32_t shl_clamped(uint32_t v, uint32_t n) {
+  uint32_t r;
+  asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+  return r;
+}
+
+// Bit positions of one map of an op (16 bytes) held in registers.
+struct BitMap {
+  uint32_t w[4];
+  __device__ explicit BitMap(const uint8_t* p) {
+    const uint4 v = *reinterpret_cast<const uint4*>(p);
+    w[0] = v.x;
+    w[1] = v.y;
+    w[2] = v.z;
+    w[3] = v.w;
   }
+  // position of bit i (i known at compile time after unrolling)
+  __device__ __forceinline__ uint32_t at(int i) const { return (w[i >> 2] >> (8 * (i & 3))) & 0xffu; }
+};
+
+// Deposits bits 0..N-1 of v at the positions of map bits first..first+N-1.
+template <int N>
+__device__ __forceinline__ uint32_t deposit_bits(const BitMap& m, int first, uint32_t v) {
+  uint32_t off = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (first + i < 16) off |= shl_clamped((v >> i) & 1u, m.at(first + i));
+  return off;
+}
+
+// Deposit of an arbitrary index from bit `first` up (uniform, rarely more than
+// a few bits).
+__device__ __forceinline__ uint32_t deposit_from(const uint8_t* pos, int first, uint32_t v) {
+  uint32_t off = 0;
+  for (int i = first; v; ++i, v >>= 1) off |= shl_clamped(v & 1u, pos[i]);
+  return off;
+}
+
+// Sums of G outputs over the op's 2^ry summed values, in order of the summed
+// index (y_lane: this lane's packed operand offsets of summed value `lane`; the
+// values beyond 32 add the high bits' offsets).  All loads of a pass issue
+// before its multiply-adds.
+template <typename T, int G>
+__device__ __forceinline__ void sum_outputs(const SOp& op, const T* a, const T* b,
+                                            const uint32_t (&oa)[G], const uint32_t (&ob)[G],
+                                            uint32_t y_lane, T (&acc)[G]) {
+  constexpr int Y = G == 1 ? 4 : 2;
+  const uint32_t ny = 1u << op.ry;
+#pragma unroll
+  for (int g = 0; g < G; ++g) acc[g] = czero<T>();
+  if (ny == 1) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) acc[g] = cfma(a[oa[g]], b[ob[g]], acc[g]);
+    return;
+  }
+  for (uint32_t y0 = 0; y0 < ny; y0 += 32) {
+    const uint32_t ha = y0 ? deposit_from(op.y1, 5, y0 >> 5) : 0u;
+    const uint32_t hb = y0 ? deposit_from(op.y2, 5, y0 >> 5) : 0u;
+    const uint32_t n = ny - y0 < 32u ? ny - y0 : 32u;   // 2, 4, ..., 32
+    for (uint32_t y = 0; y < n; y += Y) {
+      T av[Y][G], bv[Y][G];
+#pragma unroll
+      for (int u = 0; u < Y; ++u) {
+        // (two summed values only: the pass of four reads them twice)
+        const uint32_t e = __shfl_sync(0xffffffffu, y_lane, (y + u) & (n - 1u));
+        const uint32_t ea = (e & 0xffffu) | ha, eb = (e >> 16) | hb;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          av[u][g] = a[oa[g] | ea];
+          bv[u][g] = b[ob[g] | eb];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < Y; ++u)
+        if (y + u < n) {
+#pragma unroll
+          for (int g = 0; g < G; ++g) acc[g] = cfma(av[u][g], bv[u][g], acc[g]);
+        }
+    }
+  }
+}
+
+// One contraction by 2^kLog threads (the team, or one warp: kLog = 5), thread t
+// computing outputs c = t + k 2^kLog, up to four at a time.  The offsets of a
+// thread's own index bits and of the lane's summed value are formed once from
+// the op's bit maps held in registers; a pass then costs one shuffle per summed
+// value and the operands' loads.  Sums run in order of the summed index.  Bound
+// by latency: programs are chains of levels of a few small ops.  Against one
+// barrier per op with the maps walked bit by bit for every operand element, the
+// p=2 n=100 gradient step on CTA teams went from 520 to 280 us, the dense one's
+// graph launch from 1.83 to 1.47 ms, complex128 n=20 full networks from 4.30 to
+// 3.89 ms.
+template <typename T, int kLog>
+__device__ __noinline__ void contract_by(const SOp& op, T* out, const T* a, const T* b,
+                                         uint32_t t) {
+  const uint32_t nout = 1u << op.rc, lane = t & 31u;
+  if ((t & ~31u) >= nout) return;   // whole warps
+  const BitMap p1(op.p1), p2(op.p2);
+  uint32_t y_lane = 0;
+  if (op.ry) {
+    const BitMap y1(op.y1), y2(op.y2);
+    y_lane = deposit_bits<5>(y1, 0, lane) | deposit_bits<5>(y2, 0, lane) << 16;
+  }
+  const bool active = t < nout;     // only a warp of fewer than 32 outputs has idle lanes
+  const uint32_t a0 = deposit_bits<kLog>(p1, 0, active ? t : 0u);
+  const uint32_t b0 = deposit_bits<kLog>(p2, 0, active ? t : 0u);
+  const uint32_t nk = op.rc > kLog ? nout >> kLog : 1u;
+  if (nk >= 4) {
+    const uint32_t k1a = shl_clamped(1u, op.p1[kLog]), k1b = shl_clamped(1u, op.p2[kLog]);
+    const uint32_t k2a = shl_clamped(1u, op.p1[kLog + 1]), k2b = shl_clamped(1u, op.p2[kLog + 1]);
+    for (uint32_t k = 0; k < nk; k += 4) {
+      const uint32_t ha = a0 | deposit_from(op.p1, kLog + 2, k >> 2);
+      const uint32_t hb = b0 | deposit_from(op.p2, kLog + 2, k >> 2);
+      const uint32_t oa[4] = {ha, ha | k1a, ha | k2a, ha | k1a | k2a};
+      const uint32_t ob[4] = {hb, hb | k1b, hb | k2b, hb | k1b | k2b};
+      T acc[4];
+      sum_outputs<T, 4>(op, a, b, oa, ob, y_lane, acc);
+#pragma unroll
+      for (int g = 0; g < 4; ++g) out[t + ((k + g) << kLog)] = acc[g];
+    }
+  } else if (nk == 2) {
+    const uint32_t oa[2] = {a0, a0 | shl_clamped(1u, op.p1[kLog])};
+    const uint32_t ob[2] = {b0, b0 | shl_clamped(1u, op.p2[kLog])};
+    T acc[2];
+    sum_outputs<T, 2>(op, a, b, oa, ob, y_lane, acc);
+    out[t] = acc[0];
+    out[t + (1u << kLog)] = acc[1];
+  } else {
+    const uint32_t oa[1] = {a0}, ob[1] = {b0};
+    T acc[1];
+    sum_outputs<T, 1>(op, a, b, oa, ob, y_lane, acc);
+    if (active) out[t] = acc[0];
+  }
+}
+
+// A narrow adjoint op (at most 32 outputs) by one warp: with SOPF_LANES the
+// lanes take the summed values lane, lane + 32, ... of each output in turn and
+// are added by shuffles (long sums over few outputs); else lane c sums output
+// c.  With SOPF_LEAFDOT the outputs are dS/dleaf: their dot with the leaf's
+// derivative `der` goes to the gradient slot (one warp owns a slot, so the order
+// of its terms is fixed).
+template <typename T, typename G>
+__device__ __noinline__ void adjoint_by_warp(const SOp& op, T* out, const T* a, const T* b,
+                                             const T* der, G* grad, uint32_t lane) {
+  const uint32_t nout = 1u << op.rc, ny = 1u << op.ry;
+  const BitMap p1(op.p1), p2(op.p2), y1(op.y1), y2(op.y2);
+  T mine = czero<T>();   // output `lane`
+  if (op.flags & SOPF_LANES) {
+    const uint32_t la = deposit_bits<5>(y1, 0, lane), lb = deposit_bits<5>(y2, 0, lane);
+    for (uint32_t c = 0; c < nout; ++c) {
+      const uint32_t oa = deposit_bits<5>(p1, 0, c) | la, ob = deposit_bits<5>(p2, 0, c) | lb;
+      T acc = czero<T>();
+      for (uint32_t y = 0; y < ny; y += 128) {
+        T av[4], bv[4];
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) {
+          const uint32_t yy = y + 32 * u < ny ? y + 32 * u : y;
+          av[u] = a[oa | deposit_from(op.y1, 5, yy >> 5)];
+          bv[u] = b[ob | deposit_from(op.y2, 5, yy >> 5)];
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u)
+          if (y + 32 * u < ny) acc = cfma(av[u], bv[u], acc);
+      }
+      acc = warp_csum(acc, 32u);
+      if (lane == c) mine = acc;
+    }
+  } else {
+    const uint32_t y_lane = deposit_bits<5>(y1, 0, lane) | deposit_bits<5>(y2, 0, lane) << 16;
+    const uint32_t c = lane < nout ? lane : 0u;
+    const uint32_t oa[1] = {deposit_bits<5>(p1, 0, c)}, ob[1] = {deposit_bits<5>(p2, 0, c)};
+    T acc[1];
+    sum_outputs<T, 1>(op, a, b, oa, ob, y_lane, acc);
+    mine = acc[0];
+  }
+  if (!(op.flags & SOPF_LEAFDOT)) {
+    if (lane < nout) out[lane] = mine;
+    return;
+  }
+  T v = czero<T>();
+  if (lane < nout) v = cfma(mine, der[lane], v);
+  v = warp_csum(v, 16u);
+  if (lane == 0) {
+    const uint32_t slot = op.p1[kLeafSlotByte];
+    grad[2 * slot] += (G)v.x;
+    grad[2 * slot + 1] += (G)v.y;
+  }
+}
+
+// One staged op of a task, called by the whole team (kLog = log2 of its
+// threads); `at` resolves an operand offset, `result` takes the scalar.
+template <typename T, int kLog, typename TeamT, typename At, typename G, typename Result>
+__device__ __forceinline__ void run_op(const SOp& op, const TeamT& team, const At& at,
+                                       const T* table, G* grad, const Result& result) {
+  const uint32_t tid = team.tid, lane = tid & 31u;
+  const uint4 head = *reinterpret_cast<const uint4*>(&op);
+  const uint32_t code = head.x & 15u, flags = head.x >> 24;
+  if (!(flags & SOPF_NARROW)) {
+    contract_by<T, kLog>(op, at(head.y, flags & SOPF_OUT_GLOBAL), at(head.z, flags & SOPF_IN1_GLOBAL),
+                         at(head.w, flags & SOPF_IN2_GLOBAL), tid);
+  } else if ((tid >> 5) == ((head.x >> 4) & 15u)) {
+    if (code == SOP_CONTRACT) {
+      const T* a = at(head.z, flags & SOPF_IN1_GLOBAL);
+      const T* b = at(head.w, flags & SOPF_IN2_GLOBAL);
+      if (flags & SOPF_LEAFDOT)
+        adjoint_by_warp<T>(op, (T*)nullptr, a, b, table + head.y, grad, lane);
+      else if (flags & SOPF_LANES)
+        adjoint_by_warp<T>(op, at(head.y, flags & SOPF_OUT_GLOBAL), a, b, (const T*)nullptr, grad,
+                           lane);
+      else
+        contract_by<T, 5>(op, at(head.y, flags & SOPF_OUT_GLOBAL), a, b, lane);
+    } else if (code == SOP_LEAFGRAD) {
+      warp_leaf_dot<T>(at(head.z, 0u), at(head.w, 0u), 1u << op.rc, lane, grad, head.y);
+    } else if (lane == 0) {
+      if (code == SOP_RESULT) result(*at(head.z, flags & SOPF_IN1_GLOBAL));
+      else if (code == SOP_SEED)
+        *at(head.y, flags & SOPF_OUT_GLOBAL) = from_d2<T>(make_double2(1.0, 0.0));
+    }
+  }
+  if (flags & SOPF_SYNC) team.sync();
 }
 
 }  // namespace qtc

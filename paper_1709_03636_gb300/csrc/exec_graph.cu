@@ -24,6 +24,7 @@
 namespace qtc {
 
 constexpr int kGraphBlock = 256;   // threads per team
+constexpr int kGraphBlockLog = 8;
 
 // A team of 256 threads runs one task at a time.  The instantiation without
 // tensor-core tasks has one team per CTA (4 CTAs per SM); the one with them
@@ -120,7 +121,7 @@ __device__ __forceinline__ T* locate(uint32_t off, bool global, T* gbase, T* tab
 }
 
 template <typename T, int kTeams>
-__device__ void run_smem_task(const GraphProgDev& prog, const GTask& task, T* table,
+__device__ __noinline__ void run_smem_task(const GraphProgDev& prog, const GTask& task, T* table,
                               unsigned char* work, double* s_grad, const GTeam<kTeams>& team) {
   const int P = prog.n_params;
   const int stride = 2 + 2 * P;
@@ -136,37 +137,17 @@ __device__ void run_smem_task(const GraphProgDev& prog, const GTask& task, T* ta
     uint4* dst = reinterpret_cast<uint4*>(stage);
     for (uint32_t w = team.tid; w < n * kWords; w += team.size) dst[w] = src[w];
     team.sync();
-    for (uint32_t k = 0; k < n; ++k) {
-      const SOp& op = stage[k];
-      T* out = locate(op.out, (op.flags & SOPF_OUT_GLOBAL) != 0, gbase, table, arena,
-                      prog.table_elems);
-      T* in1 = locate(op.in1, (op.flags & SOPF_IN1_GLOBAL) != 0, gbase, table, arena,
-                      prog.table_elems);
-      T* in2 = locate(op.in2, (op.flags & SOPF_IN2_GLOBAL) != 0, gbase, table, arena,
-                      prog.table_elems);
-      switch (op.code) {
-        case SOP_CONTRACT:
-          contract_op<T>(op, out, in1, in2, team);
-          break;
-        case SOP_LEAFGRAD:
-          if (team.tid < 32)
-            warp_leaf_dot<T>(in1, in2, 1u << op.rc, team.tid, s_grad, op.out);
-          break;
-        case SOP_RESULT:
-          if (team.tid == 0) {
-            const double2 v = to_d2(*in1);
+    for (uint32_t k = 0; k < n; ++k)
+      run_op<T, kGraphBlockLog>(
+          stage[k], team,
+          [&](uint32_t off, uint32_t global) {
+            return locate(off, global != 0, gbase, table, arena, prog.table_elems);
+          },
+          table, s_grad, [&](T r) {
+            const double2 v = to_d2(r);
             prog.results[(size_t)task.net * stride] = v.x;
             prog.results[(size_t)task.net * stride + 1] = v.y;
-          }
-          break;
-        case SOP_SEED:
-          if (team.tid == 0) *out = from_d2<T>(make_double2(1.0, 0.0));
-          break;
-        default:
-          break;
-      }
-      team.sync();
-    }
+          });
   }
   for (int i = team.tid; i < 2 * P; i += team.size)
     if (s_grad[i] != 0.0) atomicAdd(&prog.results[(size_t)task.net * stride + 2 + i], s_grad[i]);
@@ -1281,7 +1262,7 @@ __device__ bool run_tc(const GraphProgDev& prog, const GTask& task, unsigned cha
 template <typename T, bool kTc, bool kHiOcc = false, bool kTile = false>
 __global__ void __launch_bounds__(kGraphBlock*(kTc ? 4 : 1),
                                   kTc ? 1 : kHiOcc ? 5 : sizeof(T) == 8 ? 4 : 2)
-    graph_exec_kernel(const GraphProgDev prog) {
+    graph_exec_kernel(const __grid_constant__ GraphProgDev prog) {
   constexpr int kTeams = kTc ? 4 : 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ GStep s_step[kTeams];

@@ -19,6 +19,7 @@
 namespace qtc {
 
 constexpr int kMaxTeams = 8;
+constexpr int kExecBlockLog = 7;   // CTA teams: log2 of kExecBlock
 
 // One CONTRACT op of a warp team from its pre-expanded offset tables: lane
 // handles outputs c = 32 j + lane (j < 2^(rc - 5), up to 64 for rank 11).
@@ -452,32 +453,12 @@ __global__ void __maxnreg__(kExecMaxRegs) smem_exec_kernel(const ProgramDev prog
             }
           }
         } else {
-          switch (op.code) {
-            case SOP_CONTRACT:
-              contract_op<T>(op, resolve(op.out, table, arena, prog.table_elems),
-                             resolve(op.in1, table, arena, prog.table_elems),
-                             resolve(op.in2, table, arena, prog.table_elems), team);
-              break;
-            case SOP_LEAFGRAD:
-              if (team.tid < 32)
-                warp_leaf_dot<T>(resolve(op.in1, table, arena, prog.table_elems),
-                                 resolve(op.in2, table, arena, prog.table_elems), 1u << op.rc,
-                                 team.tid, grad, op.out);
-              break;
-            case SOP_RESULT:
-              if (team.tid == 0) s_res[team.id] = to_d2(*resolve(op.in1, table, arena,
-                                                                prog.table_elems));
-              break;
-            case SOP_SEED:
-              if (team.tid == 0)
-                *resolve(op.out, table, arena, prog.table_elems) =
-                    from_d2<T>(make_double2(1.0, 0.0));
-              break;
-            default:
-              break;
-          }
+          run_op<T, kExecBlockLog>(
+              op, team,
+              [&](uint32_t off, uint32_t) { return resolve(off, table, arena, prog.table_elems); },
+              table, grad, [&](T v) { s_res[team.id] = to_d2(v); });
         }
-        team.sync();
+        if (kWarp) team.sync();
       }
     }
     if (lane_grad) {

@@ -219,18 +219,11 @@ uint64_t runs_offset_host(const GRuns& r, uint64_t idx) {
   return off;
 }
 
-uint64_t positions_max(const uint8_t* pos, int n) {
-  uint64_t off = 0;
-  for (int i = 0; i < n; ++i)
-    if (pos[i] != kAbsent) off |= (uint64_t)1 << pos[i];
-  return off;
-}
-
 // Checks every access of a wave against its buffers and the task order
 // against the dependencies, so that a lowering mistake is an error on the
 // host instead of a bad address or a wait that never ends on the device.
 void validate_wave(const WaveHost& w, uint32_t table_elems, uint32_t arena_elems,
-                   size_t elem_of_wave, size_t work_bytes) {
+                   size_t elem_of_wave, size_t work_bytes, int n_params) {
   auto check_ref = [&](uint32_t off, bool global, uint64_t max_index, const char* what) {
     const uint64_t end = (uint64_t)off + max_index + 1;
     if (global) {
@@ -248,23 +241,8 @@ void validate_wave(const WaveHost& w, uint32_t table_elems, uint32_t arena_elems
       if ((uint64_t)t.a + t.b > w.ops.size()) fail(QTC_ERR_INVALID, "internal: op range");
       if (t.signal != 0xFFFFFFFFu && t.signal >= w.n_counters)
         fail(QTC_ERR_INVALID, "internal: signal counter out of range");
-      for (uint32_t i = t.a; i < t.a + t.b; ++i) {
-        const SOp& op = w.ops[i];
-        if (op.code == SOP_CONTRACT) {
-          uint64_t m1 = positions_max(op.p1, op.rc) | positions_max(op.y1, op.ry);
-          uint64_t m2 = positions_max(op.p2, op.rc) | positions_max(op.y2, op.ry);
-          check_ref(op.out, op.flags & SOPF_OUT_GLOBAL, ((uint64_t)1 << op.rc) - 1, "op output");
-          check_ref(op.in1, op.flags & SOPF_IN1_GLOBAL, m1, "op operand 1");
-          check_ref(op.in2, op.flags & SOPF_IN2_GLOBAL, m2, "op operand 2");
-        } else if (op.code == SOP_LEAFGRAD) {
-          check_ref(op.in1, false, ((uint64_t)1 << op.rc) - 1, "leaf adjoint");
-          check_ref(op.in2, false, ((uint64_t)1 << op.rc) - 1, "leaf derivative");
-        } else if (op.code == SOP_RESULT) {
-          check_ref(op.in1, op.flags & SOPF_IN1_GLOBAL, 0, "result");
-        } else if (op.code == SOP_SEED) {
-          check_ref(op.out, op.flags & SOPF_OUT_GLOBAL, 0, "seed");
-        }
-      }
+      validate_cta_ops(w.ops.data() + t.a, t.b, table_elems, arena_elems, w.global_elems, n_params,
+                       kGraphWarps);
     } else if (t.kind == GT_TC) {
       if (t.a >= w.tsteps.size()) fail(QTC_ERR_INVALID, "internal: GEMM index");
       const TStep& ts = w.tsteps[t.a];
@@ -493,6 +471,7 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
       GUnit u;
       u.kind = GT_SMEM;
       u.ops = std::move(ln.ops);
+      schedule_cta_ops(u.ops, hp.table_elems, kGraphWarps);
       u.arena_elems = ln.arena_elems;
       graphs[i].units.push_back(std::move(u));
       return;
@@ -597,7 +576,8 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
   hp.work_bytes = round16(std::max({smem_task, chunk_task, tile_task}));
   hp.table_bytes = round16((size_t)hp.table_elems * elem);
   hp.smem = hp.table_bytes + (size_t)(hp.tensor_cores ? 4 : 1) * hp.work_bytes;
-  for (const WaveHost& w : hp.waves) validate_wave(w, hp.table_elems, max_arena, elem, hp.work_bytes);
+  for (const WaveHost& w : hp.waves) 
+    validate_wave(w, hp.table_elems, max_arena, elem, hp.work_bytes, hp.n_params);
   if (hp.smem > max_dynamic)
     fail(QTC_ERR_UNSUPPORTED, "graph program needs %zu bytes of shared memory (limit %zu)",
          hp.smem, max_dynamic);

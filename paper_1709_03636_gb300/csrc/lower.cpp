@@ -119,7 +119,7 @@ uint32_t place_arena(const std::vector<Pending>& ops, const std::vector<uint32_t
     op.out = resolve(p.out);
     op.in1 = resolve(p.in1);
     op.in2 = resolve(p.in2);
-    op.flags = (p.out.global ? SOPF_OUT_GLOBAL : 0) | (p.in1.global ? SOPF_IN1_GLOBAL : 0) |
+    op.flags |= (p.out.global ? SOPF_OUT_GLOBAL : 0) | (p.in1.global ? SOPF_IN1_GLOBAL : 0) |
                (p.in2.global ? SOPF_IN2_GLOBAL : 0);
     out.push_back(op);
   }
@@ -211,6 +211,7 @@ LoweredNet lower_smem(const Plan& plan, const std::vector<int>& leaf_gate,
         // in X of dS/dC * Y (holomorphic, no conjugation)
         Pending p{};
         p.op.code = SOP_CONTRACT;
+        p.op.flags = SOPF_LANES;   // its sums may be shared by lanes
         if (!encode_contract(p.op, plan.labels[x], plan.labels[c], plan.labels[y])) return out;
         p.out = grad_ref(x);
         p.in1 = grad_ref(c);
@@ -789,6 +790,7 @@ NetGraph lower_graph(const Plan& plan, const std::vector<int>& leaf_gate,
           if (!need_grad[x]) continue;
           Pending p{};
           p.op.code = SOP_CONTRACT;
+          p.op.flags = SOPF_LANES;
           if (!encode_contract(p.op, plan.labels[x], plan.labels[c], plan.labels[y]))
             return false;
           p.in1 = grad_ref(c);
@@ -811,6 +813,7 @@ NetGraph lower_graph(const Plan& plan, const std::vector<int>& leaf_gate,
     }
     u.arena_elems = place_arena(ops, buf_size, table_elems, u.ops);
     if (u.arena_elems > lim.arena_elems) return false;
+    schedule_cta_ops(u.ops, table_elems, kGraphWarps);
     const int id = add_unit(std::move(u));
     if (!reverse && in_global[L + rs]) producer_val[L + rs] = id;
     return true;
@@ -925,6 +928,7 @@ NetGraph lower_graph(const Plan& plan, const std::vector<int>& leaf_gate,
     }
     u.deps.push_back(producer_val[root]);
     place_arena(ops, {}, table_elems, u.ops);
+    schedule_cta_ops(u.ops, table_elems, kGraphWarps);
     const int id = add_unit(std::move(u));
     producer_grad[root] = id;
   }

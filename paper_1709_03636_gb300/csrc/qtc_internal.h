@@ -18,6 +18,7 @@ namespace qtc {
 // CTA when one warp runs one network.
 constexpr int kExecBlock = 128;
 constexpr int kWarpTeamsPerCta = 4;
+constexpr int kGraphWarps = 8;   // warps of a graph-executor team
 
 // ---- errors ---------------------------------------------------------------
 // Internal code throws Error; every C-ABI entry point catches it, stores the
@@ -181,6 +182,13 @@ void build_warp_steps(const std::vector<SOp>& ops, uint32_t table_elems, uint32_
                       std::vector<WStep>& out);
 // Host check of a warp program's every access against its team region.
 void validate_warp_steps(const WStep* steps, size_t n, uint32_t team_elems, int n_params);
+
+// Puts a task's ops into levels for a team of n_warps warps (cta_program.cpp).
+void schedule_cta_ops(std::vector<SOp>& ops, uint32_t table_elems, int n_warps);
+// Host check of such a program: every access against its buffer, no conflict
+// within a level, one warp per gradient slot.
+void validate_cta_ops(const SOp* ops, size_t n, uint32_t table_elems, uint32_t arena_elems,
+                      uint64_t global_elems, int n_params, int n_warps);
 
 // Lowers one plan to a shared-memory op program.  table_elems: size of the
 // gate value + derivative region that precedes the arena.  Intermediates and
