@@ -560,7 +560,204 @@ __global__ void __launch_bounds__(kSvThreads, 2) sv_tile_kernel(const SvArgs a) 
   }
 }
 
-// <Z_a Z_b> for edges [e0, e0 + 16): one pass over the state.
+// ---- <Z_a Z_b> of every edge in one pass over the state ----------------------
+//
+// Signed sums of p(x) = |psi_x|^2.  A tile is 2^12 consecutive amplitudes: lanes
+// are bits 0..4, a thread's 16 registers bits 5..8, its warp bits 9..11.  A
+// thread forms the signed sums of its 16 values over every subset of at most two
+// register bits (a pruned Walsh-Hadamard transform); an edge inside the tile
+// bits is one of these with the signs of its lane and warp bits, so they are
+// accumulated over all tiles and signed once per CTA.  An edge with one end
+// above the tile bits needs that end's sign per tile: a tile's 12 one-bit sums
+// and its total are left in the first amplitudes of the tile itself (read for
+// the last time here; the state is internal), and a second launch adds them up
+// per edge.
+//
+// GB300's FP64 pipe does two operations per clock and SM, and that is what
+// bound the former form (16 FP64 sums per amplitude and launch, m / 16
+// launches): n = 21 with 63 edges, depth 3, 654 -> 150 us in all.  complex64
+// states are summed as pairs of floats (exact products and error-free
+// additions, about 48 bits; the values agree to every float32 bit) on the FP32
+// pipe instead; complex128 in FP64, about ten operations per amplitude for all
+// edges.
+constexpr int kZzBits = 12, kZzThreads = 256;
+
+struct FloatPair {
+  float h, l;
+};
+__device__ __forceinline__ FloatPair pair_sum(float a, float al, float b, float bl) {
+  const float s = a + b, t = s - a;
+  const float e = ((a - (s - t)) + (b - t)) + (al + bl);
+  const float h = s + e;
+  return {h, e - (h - s)};
+}
+__device__ __forceinline__ FloatPair zadd(FloatPair a, FloatPair b) {
+  return pair_sum(a.h, a.l, b.h, b.l);
+}
+__device__ __forceinline__ FloatPair zsub(FloatPair a, FloatPair b) {
+  return pair_sum(a.h, a.l, -b.h, -b.l);
+}
+__device__ __forceinline__ double zadd(double a, double b) { return a + b; }
+__device__ __forceinline__ double zsub(double a, double b) { return a - b; }
+__device__ __forceinline__ FloatPair zprob(float2 v) {
+  const float x = v.x * v.x, y = v.y * v.y;
+  return pair_sum(x, fmaf(v.x, v.x, -x), y, fmaf(v.y, v.y, -y));
+}
+__device__ __forceinline__ double zprob(double2 v) { return v.x * v.x + v.y * v.y; }
+__device__ __forceinline__ FloatPair zshfl(FloatPair v, int m) {
+  return {__shfl_xor_sync(0xffffffffu, v.h, m), __shfl_xor_sync(0xffffffffu, v.l, m)};
+}
+__device__ __forceinline__ double zshfl(double v, int m) {
+  return __shfl_xor_sync(0xffffffffu, v, m);
+}
+__device__ __forceinline__ double zdouble(FloatPair v) { return (double)v.h + (double)v.l; }
+__device__ __forceinline__ double zdouble(double v) { return v; }
+
+template <typename T> struct ZzOf;
+template <> struct ZzOf<float2> { using type = FloatPair; };
+template <> struct ZzOf<double2> { using type = double; };
+
+template <typename T>
+__global__ void __launch_bounds__(kZzThreads) sv_zz_kernel(T* psi, int n, int m, const int2* edges,
+                                                           double* acc) {
+  using S = typename ZzOf<T>::type;
+  // sums over subsets of register bits: none, {i}, {i, j} (i < j)
+  constexpr int kSums = 11;
+  __shared__ double s_sum[kSums][kZzThreads];
+  __shared__ double s_warp[kZzThreads / 32][10];
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint64_t n_tiles = 1ull << (n - kZzBits);
+  S total[kSums];
+#pragma unroll
+  for (int k = 0; k < kSums; ++k) total[k] = S{};
+  for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    T* at = psi + (tile << kZzBits);
+    S p[16];
+    {
+      T v[16];
+#pragma unroll
+      for (int r = 0; r < 16; ++r) v[r] = at[(warp << 9) | (r << 5) | lane];
+#pragma unroll
+      for (int r = 0; r < 16; ++r) p[r] = zprob(v[r]);
+    }
+    // one[i] = sum of p signed by register bit i, two[] by pairs of bits; each
+    // step folds the lowest remaining bit away
+    S one[4], two[6];
+    int k2 = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int half = 8 >> i;
+      S d[8];
+#pragma unroll
+      for (int r = 0; r < half; ++r) {
+        d[r] = zsub(p[2 * r], p[2 * r + 1]);
+        p[r] = zadd(p[2 * r], p[2 * r + 1]);
+      }
+      // the differences folded further: signed by bit i and by one later bit
+      int rest = half;
+#pragma unroll
+      for (int j = i + 1; j < 4; ++j) {
+        S t = zsub(d[0], d[1]);
+#pragma unroll
+        for (int r = 1; r < 4; ++r)
+          if (2 * r < rest) t = zadd(t, zsub(d[2 * r], d[2 * r + 1]));
+        two[k2++] = t;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (2 * r < rest) d[r] = zadd(d[2 * r], d[2 * r + 1]);
+        rest >>= 1;
+      }
+      one[i] = d[0];
+    }
+    total[0] = zadd(total[0], p[0]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) total[1 + i] = zadd(total[1 + i], one[i]);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) total[5 + k] = zadd(total[5 + k], two[k]);
+    // the tile's one-bit sums and total (only edges above the tile bits use
+    // them): p[0] over the lanes as a Walsh-Hadamard transform, lane l ending
+    // with the sum signed by subset l of the lane bits
+    if (n > kZzBits) {
+      S w = p[0];
+#pragma unroll
+      for (int q = 0; q < 5; ++q) {
+        const S o = zshfl(w, 1 << q);
+        w = ((lane >> q) & 1u) ? zsub(o, w) : zadd(w, o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) one[i] = zadd(one[i], zshfl(one[i], 1 << q));
+      }
+      const int slot = lane == 0 ? 0 : (lane & (lane - 1)) == 0 ? 32 - __clz(lane) : -1;
+      __syncthreads();   // every thread has read the tile; s_warp is free
+      if (slot >= 0) s_warp[warp][slot] = zdouble(w);   // total, lane bits 0..4
+      if (lane < 4) {
+        const S o = lane == 0 ? one[0] : lane == 1 ? one[1] : lane == 2 ? one[2] : one[3];
+        s_warp[warp][6 + lane] = zdouble(o);
+      }
+      __syncthreads();
+      if (threadIdx.x < 13) {
+        // 0: total; 1 + a: signed by tile bit a
+        const int a = (int)threadIdx.x - 1;
+        double s = 0.0;
+        for (int u = 0; u < kZzThreads / 32; ++u) {
+          const double v = s_warp[u][a < 5 ? a + 1 : a < 9 ? a + 1 : 0];
+          s += a >= 9 && ((u >> (a - 9)) & 1) ? -v : v;
+        }
+        reinterpret_cast<double*>(at)[threadIdx.x] = s;
+      }
+    }
+  }
+  // edges inside the tile bits
+#pragma unroll
+  for (int k = 0; k < kSums; ++k) s_sum[k][threadIdx.x] = zdouble(total[k]);
+  __syncthreads();
+  for (int e = warp; e < m; e += kZzThreads / 32) {
+    const int2 ed = edges[e];
+    if (ed.x >= kZzBits || ed.y >= kZzBits) continue;
+    const uint32_t mask = (1u << ed.x) | (1u << ed.y), reg = (mask >> 5) & 15u;
+    const uint32_t thr = (mask & 31u) | ((mask >> 9) << 5);   // thread index bits in the sign
+    int k = 0;
+    if (reg) {
+      const int i = __ffs(reg) - 1, j = 31 - __clz(reg);
+      // {i} -> 1 + i; {i, j}: pairs (0,1) (0,2) (0,3) (1,2) (1,3) (2,3) -> 5..10
+      k = i == j ? 1 + i : 5 + (i == 0 ? j - 1 : i == 1 ? j + 1 : 5);
+    }
+    double s = 0.0;
+    for (uint32_t t = lane; t < kZzThreads; t += 32) {
+      const double v = s_sum[k][t];
+      s += (__popc(t & thr) & 1) ? -v : v;
+    }
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) atomicAdd(&acc[1 + e], s);
+  }
+}
+
+// Edges with an end above the tile bits: one CTA per edge adds the tiles' sums
+// with that end's sign (both ends above: the totals).
+template <typename T>
+__global__ void __launch_bounds__(kZzThreads) sv_zz_tiles_kernel(const T* psi, int n,
+                                                                 const int2* edges, double* acc) {
+  __shared__ double s_part[kZzThreads / 32];
+  const int2 ed = edges[blockIdx.x];
+  const int lo = min(ed.x, ed.y), hi = max(ed.x, ed.y);
+  if (hi < kZzBits) return;
+  const uint64_t n_tiles = 1ull << (n - kZzBits);
+  const uint64_t sign = (1ull << (hi - kZzBits)) | (lo >= kZzBits ? 1ull << (lo - kZzBits) : 0ull);
+  const int slot = lo >= kZzBits ? 0 : 1 + lo;
+  double s = 0.0;
+  for (uint64_t t = threadIdx.x; t < n_tiles; t += kZzThreads) {
+    const double v = reinterpret_cast<const double*>(psi + (t << kZzBits))[slot];
+    s += (__popcll(t & sign) & 1) ? -v : v;
+  }
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kZzThreads / 32; ++w) s += s_part[w];
+    acc[1 + blockIdx.x] = s;
+  }
+}
+
+// <Z_a Z_b> for edges [e0, e0 + 16) of a state of fewer than 2^12 amplitudes.
 template <typename T>
 __global__ void __launch_bounds__(256) sv_edge_kernel(void* psi_v, int n, int m,
                                                       const int2* edges, double* acc, int e0) {
@@ -662,9 +859,24 @@ static cudaError_t sv_launch_t(void* psi, int n, int m, const uint32_t* adj_dev,
       err = cudaGetLastError();
       if (err != cudaSuccess) return err;
     }
-  if (per_edge)
+  if (per_edge && n >= kZzBits) {
+    const unsigned tiles = (unsigned)(1ull << (n - kZzBits));
+    // two CTAs per SM: each thread has 16 loads in flight
+    sv_zz_kernel<T><<<std::min<unsigned>(tiles, 2u * (unsigned)sms), kZzThreads, 0, stream>>>(
+        reinterpret_cast<T*>(psi), n, m, edges_dev, acc_dev);
+    ++*launches;
+    err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+    if (n > kZzBits) {
+      sv_zz_tiles_kernel<T><<<m, kZzThreads, 0, stream>>>(reinterpret_cast<const T*>(psi), n,
+                                                          edges_dev, acc_dev);
+      ++*launches;
+      err = cudaGetLastError();
+      if (err != cudaSuccess) return err;
+    }
+  } else if (per_edge)
     for (int e0 = 0; e0 < m; e0 += 16) {
-      sv_edge_kernel<T><<<1024, 256, 0, stream>>>(psi, n, m, edges_dev, acc_dev, e0);
+      sv_edge_kernel<T><<<1, 256, 0, stream>>>(psi, n, m, edges_dev, acc_dev, e0);
       ++*launches;
       err = cudaGetLastError();
       if (err != cudaSuccess) return err;

@@ -82,3 +82,18 @@ def test_statevector_device_form_and_tensor_network_agree(engine):
     C, per_edge, _ = q.qaoa_expectation(engine, batch, g, b, "c64")
     assert abs(C - out[0].item()) < 1e-5 * ref
     assert np.max(np.abs(np.array(per_edge) - out[1:].cpu().numpy())) < 4e-6
+
+
+@pytest.mark.parametrize("n,d,p", [(11, 4, 1), (12, 5, 2), (13, 6, 1), (14, 9, 2), (17, 8, 1)])
+@pytest.mark.parametrize("dtype,tol", [("c128", 1e-11), ("c64", 2e-6)])
+def test_statevector_per_edge_around_the_tile_size(engine, n, d, p, dtype, tol):
+    """Per-edge values below, at and above one tile of 2^12 amplitudes, with
+    edges inside the tile bits, across them and above them."""
+    edges = [tuple(sorted(e)) for e in random_regular_graph(n, d if n * d % 2 == 0 else d + 1, n)]
+    edges = sorted(set(edges) | {(0, n - 1), (n - 2, n - 1), (0, 1), (4, 5), (8, 9)})
+    g, b = [0.35 + 0.2 * k for k in range(p)], [0.7 - 0.3 * k for k in range(p)]
+    C, zz = q.statevector_expectation(engine, q.Circuit.qaoa(n, edges, p), g, b, dtype,
+                                      per_edge=True)
+    ref = sv.edge_zz(n, edges, g, b)
+    assert np.max(np.abs(np.array(zz) - ref)) < tol
+    assert abs(C - np.sum((1 - ref) / 2)) < tol * len(edges)
