@@ -335,7 +335,6 @@ extern "C" qtc_status qtc_selftest_wait_timeout(qtc_engine* e, void* stream) {
     d.wait_limit_ns = (long long)(e->wait_limit_ms * 1e6);
     d.table_bytes = 0;
     d.arena_bytes = 0;
-    d.stage_ops = 1;
     cuda_check(cudaMemsetAsync(cnt, 0, sizeof(unsigned int) * ctr_words(1), s), "clear");
     int per_sm = 0;
     const size_t max_dyn = max_dynamic_smem(e->smem_optin);
@@ -881,9 +880,7 @@ const HostProgram& qtc::host_program(qtc_batch* b, int dtype, int want_grad,
   // Networks of rank <= 11 whose ops sum over <= 8 labels may run one per
   // warp (warp programs); the others use the whole CTA, which stages its op
   // list in chunks.
-  uint32_t max_ops = 1;
   int max_rank = 0;
-  for (const TaskDev& t : hp->tasks) max_ops = std::max(max_ops, t.op_count);
   for (const Plan& pl : b->plans) max_rank = std::max(max_rank, pl.max_rank);
   auto round16 = [](size_t x) { return (uint32_t)((x + 15) & ~size_t(15)); };
   // warp teams need every op within the pre-expanded tables, and every
@@ -903,11 +900,12 @@ const HostProgram& qtc::host_program(qtc_batch* b, int dtype, int want_grad,
     hp->stream_steps = warp && stage == 0;
     hp->n_teams = warp ? teams : 1;
     hp->block = warp ? 32 * teams : kExecBlock;
-    hp->stage_ops = stage;
-    const size_t op_bytes = warp ? sizeof(WStep) : sizeof(SOp);
+    hp->stage_ops = warp ? stage : 0;
+    hp->half_units = warp ? 0 : stage;
     hp->table_bytes = warp ? 0 : round16((size_t)table_elems * elem);
-    const size_t lane_grad = (warp && want_grad && P <= kWarpLaneGradSlots) ? (size_t)P * 32 : 0;
-    hp->team_bytes = round16((size_t)stage * op_bytes +
+    const bool lane_sums = warp ? want_grad && P <= kWarpLaneGradSlots : hp->lane_dots;
+    const size_t lane_grad = lane_sums ? (size_t)P * 32 : 0;
+    hp->team_bytes = round16((warp ? (size_t)stage * sizeof(WStep) : (size_t)stage * 32) +
                              (lane_grad + hp->max_arena + (warp ? table_elems : 0)) * elem);
     hp->smem = hp->table_bytes + (size_t)hp->n_teams * hp->team_bytes;
     return hp->smem <= max_dynamic;
@@ -1029,22 +1027,49 @@ const HostProgram& qtc::host_program(qtc_batch* b, int dtype, int want_grad,
   } else {
     hp->max_arena = shared_arena;
   }
-  if (!ok) ok = try_layout(false, std::min<uint32_t>(max_ops, 64));
+  if (!ok) {
+    // CTA teams: a stage of twice 512 to 8 units, the largest that leaves as
+    // many CTAs on an SM as the smallest
+    auto ctas = [&] { return sm_smem / (hp->smem + 8192); };
+    hp->lane_dots = want_grad && P <= kLaneDotSlots;
+    ok = layout(false, 8);
+    if (!ok && hp->lane_dots) {
+      hp->lane_dots = false;
+      ok = layout(false, 8);
+    }
+    const size_t resident = ok ? ctas() : 0;
+    for (uint32_t half = 512; ok && half > 8; half /= 2)
+      if (layout(false, half) && ctas() >= resident) break;
+    if (ok && !layout(false, hp->half_units)) ok = layout(false, 8);
+  }
   if (!ok)
     fail(QTC_ERR_UNSUPPORTED, "program needs %zu bytes of shared memory (limit %zu)", hp->smem,
          max_dynamic);
   if (!hp->warp_teams) {
-    std::vector<SOp> all;
-    for (TaskDev& t : hp->tasks) {
-      std::vector<SOp> ops(hp->ops.begin() + t.op_begin,
-                           hp->ops.begin() + t.op_begin + t.op_count);
-      schedule_cta_ops(ops, table_elems, hp->block / 32);
-      validate_cta_ops(ops.data(), ops.size(), table_elems, hp->max_arena, 0, P, hp->block / 32);
-      t.op_begin = (uint32_t)all.size();
-      t.op_count = (uint32_t)ops.size();
-      all.insert(all.end(), ops.begin(), ops.end());
+    std::vector<std::vector<SOp>> progs;
+    size_t raw = 0;
+    for (const TaskDev& t : hp->tasks) {
+      progs.emplace_back(hp->ops.begin() + t.op_begin, hp->ops.begin() + t.op_begin + t.op_count);
+      raw += t.op_count * sizeof(SOp);
+      schedule_cta_ops(progs.back(), table_elems, kExecBlock / 32);
+      validate_cta_ops(progs.back().data(), progs.back().size(), table_elems, t.arena_elems, 0, P,
+                       kExecBlock / 32);
     }
-    hp->ops = std::move(all);
+    hp->ops.clear();
+    for (const auto& p : progs) hp->ops.insert(hp->ops.end(), p.begin(), p.end());
+    // lanes take more memory than records for the wider ops: not where that
+    // could outgrow an arena (or the static scratch array) that held the ops
+    for (uint32_t limit : {kLaneLimit, kLaneLimitSmall}) {
+      hp->stream.clear();
+      for (size_t i = 0; i < progs.size(); ++i) {
+        TaskDev& t = hp->tasks[i];
+        t.op_begin = (uint32_t)hp->stream.size();
+        t.op_count = build_cta_stream(progs[i], hp->half_units, limit, hp->lane_dots, hp->stream);
+        validate_cta_stream(hp->stream.data() + t.op_begin, hp->stream.size() - t.op_begin,
+                            t.op_count, hp->half_units, table_elems, t.arena_elems, P);
+      }
+      if (hp->stream.size() * sizeof(uint4) <= std::max<size_t>(raw, 1u << 20)) break;
+    }
   }
   b->host_programs.push_back(std::move(hp));
   return *b->host_programs.back();
@@ -1077,7 +1102,7 @@ static Prepared& prepare_graph(qtc_engine* e, qtc_batch* b, const HostProgram& h
     GraphProgDev d{};
     d.tasks = upload(e, w.tasks, stream, "upload tasks");
     d.n_tasks = (int)w.tasks.size();
-    d.ops = upload(e, w.ops, stream, "upload ops");
+    d.stream = upload(e, w.stream, stream, "upload task programs");
     d.steps = upload(e, w.steps, stream, "upload steps");
     d.tsteps = upload(e, w.tsteps, stream, "upload GEMM steps");
     d.waits = upload(e, w.waits, stream, "upload waits");
@@ -1118,7 +1143,7 @@ static Prepared& prepare_graph(qtc_engine* e, qtc_batch* b, const HostProgram& h
     d.table_elems = hp.table_elems;
     d.table_bytes = hp.table_bytes;
     d.arena_bytes = hp.work_bytes;
-    d.stage_ops = hp.stage_ops;
+    d.lane_dots = hp.lane_dots;
     d.gbase = nullptr;  // the engine's work buffer, set at launch
     d.n_params = P;
     d.n_nets = N;
@@ -1179,7 +1204,7 @@ static Prepared& prepare(qtc_engine* e, qtc_batch* b, int dtype, int want_grad,
   ProgramDev& d = pr.prog;
   auto* dg = (GateEntryDev*)e->alloc(sizeof(GateEntryDev) * G);
   auto* dt = (TaskDev*)e->alloc(sizeof(TaskDev) * hp.tasks.size());
-  auto* dops = (SOp*)e->alloc(sizeof(SOp) * std::max<size_t>(1, hp.ops.size()));
+  auto* dops = (uint4*)e->alloc(sizeof(uint4) * std::max<size_t>(1, hp.stream.size()));
   auto* dwsteps = (WStep*)e->alloc(sizeof(WStep) * std::max<size_t>(1, hp.wsteps.size()));
   auto* dcoef = e->alloc(std::max<size_t>(16, hp.coef.size()));
   auto* dw = (double*)e->alloc(sizeof(double) * N);
@@ -1190,8 +1215,8 @@ static Prepared& prepare(qtc_engine* e, qtc_batch* b, int dtype, int want_grad,
   auto* dcnt = (unsigned int*)e->alloc(sizeof(unsigned int) * 4);
   cuda_check(cudaMemcpyAsync(dg, hp.gates.data(), sizeof(GateEntryDev) * G, cudaMemcpyHostToDevice, stream), "upload gates");
   cuda_check(cudaMemcpyAsync(dt, hp.tasks.data(), sizeof(TaskDev) * hp.tasks.size(), cudaMemcpyHostToDevice, stream), "upload tasks");
-  if (!hp.ops.empty())
-    cuda_check(cudaMemcpyAsync(dops, hp.ops.data(), sizeof(SOp) * hp.ops.size(), cudaMemcpyHostToDevice, stream), "upload ops");
+  if (!hp.stream.empty())
+    cuda_check(cudaMemcpyAsync(dops, hp.stream.data(), sizeof(uint4) * hp.stream.size(), cudaMemcpyHostToDevice, stream), "upload programs");
   if (!hp.wsteps.empty())
     cuda_check(cudaMemcpyAsync(dwsteps, hp.wsteps.data(), sizeof(WStep) * hp.wsteps.size(),
                                cudaMemcpyHostToDevice, stream),
@@ -1211,11 +1236,13 @@ static Prepared& prepare(qtc_engine* e, qtc_batch* b, int dtype, int want_grad,
   d.table_bytes = hp.table_bytes;
   d.team_bytes = hp.team_bytes;
   d.stage_ops = hp.stage_ops;
+  d.half_units = hp.half_units;
+  d.lane_dots = hp.lane_dots;
   d.task_stride = hp.task_stride;
   d.coef = dcoef;
   d.tasks = dt;
   d.n_tasks = (int)hp.tasks.size();
-  d.ops = dops;
+  d.stream = dops;
   d.wsteps = dwsteps;
   d.n_params = P;
   d.n_nets = N;
@@ -1292,7 +1319,7 @@ extern "C" qtc_status qtc_batch_program_info(qtc_batch* b, int dtype, int want_g
     std::memset(info, 0, sizeof *info);
     info->graph = hp.graph ? 1 : 0;
     info->smem_bytes = (int)hp.smem;
-    info->stage_ops = (int)hp.stage_ops;
+    info->stage_ops = (int)(hp.warp_teams ? hp.stage_ops : 2 * hp.half_units);
     double tables = sizeof(GateEntryDev) * hp.gates.size();
     if (hp.graph) {
       info->n_waves = (int)hp.waves.size();
@@ -1301,7 +1328,7 @@ extern "C" qtc_status qtc_batch_program_info(qtc_batch* b, int dtype, int want_g
         info->n_global_steps += (int)(w.steps.size() + w.tsteps.size());
         info->n_gemm_steps += (int)w.tsteps.size();
         for (const GTask& t : w.tasks) info->n_smem_tasks += t.kind == GT_SMEM;
-        tables += sizeof(GTask) * w.tasks.size() + sizeof(SOp) * w.ops.size() +
+        tables += sizeof(GTask) * w.tasks.size() + sizeof(uint4) * w.stream.size() +
                   sizeof(GStep) * w.steps.size() + sizeof(TStep) * w.tsteps.size() +
                   sizeof(WaitDev) * w.waits.size();
       }
@@ -1312,7 +1339,7 @@ extern "C" qtc_status qtc_batch_program_info(qtc_batch* b, int dtype, int want_g
     } else {
       info->n_waves = 1;
       info->n_tasks = info->n_smem_tasks = (int)hp.tasks.size();
-      tables += sizeof(TaskDev) * hp.tasks.size() + sizeof(SOp) * hp.ops.size() +
+      tables += sizeof(TaskDev) * hp.tasks.size() + sizeof(uint4) * hp.stream.size() +
                 sizeof(WStep) * hp.wsteps.size();
       info->warp_teams = hp.warp_teams ? 1 : 0;
       info->n_ops = (int)hp.ops.size();

@@ -10,6 +10,9 @@
 // by cost, the others use the whole team.  A leaf's adjoint is fused with its
 // dot against the leaf's derivative, and adjoint sums that are long for their
 // few outputs are shared by a warp's lanes.  Forward sums keep their order.
+// The ops of up to 16 outputs and four terms, nine of ten, are then written as
+// lanes (one output each, its offsets formed here), so that a level of them is
+// one step of the team.
 #include <algorithm>
 #include <cstring>
 
@@ -151,7 +154,8 @@ void schedule_cta_ops(std::vector<SOp>& ops, uint32_t table_elems, int n_warps) 
   std::vector<double> load(n_warps);
   for (auto& members : by_level) {
     // narrow ops first, longest first, each to the warp with the least to do
-    // (leaf dots to the warp that owns their slot); then the team's ops
+    // (leaf dots to the first warp, so that the order of their terms is fixed);
+    // then the team's ops
     std::stable_sort(members.begin(), members.end(), [&](int x, int y) {
       const bool nx = in[x].flags & SOPF_NARROW, ny = in[y].flags & SOPF_NARROW;
       if (nx != ny) return nx;
@@ -162,8 +166,7 @@ void schedule_cta_ops(std::vector<SOp>& ops, uint32_t table_elems, int n_warps) 
       SOp op = in[i];
       if (op.flags & SOPF_NARROW) {
         int w = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-        if (op.code == SOP_LEAFGRAD) w = (int)(op.out % (uint32_t)n_warps);
-        else if (op.flags & SOPF_LEAFDOT) w = op.p1[kLeafSlotByte] % n_warps;
+        if (op.code == SOP_LEAFGRAD || (op.flags & SOPF_LEAFDOT)) w = 0;
         load[w] += op_cycles(op);
         op.code = (uint8_t)(op.code | w << 4);
       }
@@ -186,7 +189,6 @@ void validate_cta_ops(const SOp* ops, size_t n, uint32_t table_elems, uint32_t a
   };
   need(n == 0 || (ops[n - 1].flags & SOPF_SYNC), n, "no barrier at the end");
   size_t first = 0;   // of the current level
-  std::vector<int> slot_warp(n_params, -1);
   for (size_t k = 0; k < n; ++k) {
     const SOp& op = ops[k];
     const int code = op_code(op);
@@ -224,8 +226,7 @@ void validate_cta_ops(const SOp* ops, size_t n, uint32_t table_elems, uint32_t a
     }
     if (code == SOP_LEAFGRAD || dot) {
       need(slot >= 0 && slot < n_params, k, "gradient slot");
-      need(slot_warp[slot] < 0 || slot_warp[slot] == op.code >> 4, k, "slot shared by two warps");
-      slot_warp[slot] = op.code >> 4;
+      need((op.code >> 4) == 0, k, "leaf dot away from the first warp");
     }
     // no conflict with the level's earlier ops
     Range a[3], b[3];
@@ -240,6 +241,174 @@ void validate_cta_ops(const SOp* ops, size_t n, uint32_t table_elems, uint32_t a
     }
     if (op.flags & SOPF_SYNC) first = k + 1;
   }
+}
+
+namespace {
+
+// The small contractions of a level, one output per lane.
+bool fits_lanes(const SOp& op, uint32_t lane_limit, bool dots) {
+  if (op_code(op) != SOP_CONTRACT || !(op.flags & SOPF_NARROW) || (op.flags & SOPF_LANES) ||
+      (op.flags & (SOPF_OUT_GLOBAL | SOPF_IN1_GLOBAL | SOPF_IN2_GLOBAL)))
+    return false;
+  if (op.ry > 2 || (1u << op.rc) > lane_limit) return false;
+  if ((op.flags & SOPF_LEAFDOT) && (!dots || op.p1[kLeafSlotByte] >= kLaneDotSlots)) return false;
+  return op.out + (1u << op.rc) <= 0x10000u &&
+         op.in1 + (uint32_t)max_pos(op.p1, op.rc, op.y1, op.ry) < 0x10000u &&
+         op.in2 + (uint32_t)max_pos(op.p2, op.rc, op.y2, op.ry) < 0x10000u;
+}
+
+uint32_t spread(const uint8_t* pos, int n, uint32_t v) {
+  uint32_t off = 0;
+  for (int i = 0; i < n; ++i)
+    if (((v >> i) & 1u) && pos[i] != kAbsent) off |= 1u << pos[i];
+  return off;
+}
+
+CLane make_lane(const SOp& op, uint32_t c) {
+  CLane l{};
+  const bool dot = op.flags & SOPF_LEAFDOT;
+  l.out = (uint16_t)(op.out + c);
+  l.a = (uint16_t)(op.in1 + spread(op.p1, op.rc, c));
+  l.b = (uint16_t)(op.in2 + spread(op.p2, op.rc, c));
+  l.flags = (uint8_t)(op.ry | (dot ? CLF_DOT : CLF_STORE));
+  l.slot = dot ? op.p1[kLeafSlotByte] : (uint8_t)0;
+  if (op.ry >= 1) {
+    l.ya1 = (uint16_t)spread(op.y1, op.ry, 1);
+    l.yb1 = (uint16_t)spread(op.y2, op.ry, 1);
+  }
+  if (op.ry >= 2) {
+    l.ya2 = (uint16_t)spread(op.y1, op.ry, 2);
+    l.yb2 = (uint16_t)spread(op.y2, op.ry, 2);
+  }
+  return l;
+}
+
+}  // namespace
+
+uint32_t build_cta_stream(const std::vector<SOp>& ops, uint32_t half_units, uint32_t lane_limit,
+                          bool dots, std::vector<uint4>& out) {
+  if (ops.empty()) return 0;
+  if (half_units < 1 + kSOpUnits)
+    fail(QTC_ERR_INVALID, "internal: a stage of %u units", 2 * half_units);
+  struct Record {
+    std::vector<uint4> units;
+    bool level_end = false;
+  };
+  std::vector<Record> records;
+  const uint32_t max_lanes = std::min(half_units - 2, 1024u);
+  auto unit_of = [](const void* p) {
+    uint4 u;
+    std::memcpy(&u, p, sizeof u);
+    return u;
+  };
+  for (size_t first = 0; first < ops.size();) {
+    size_t last = first;
+    while (!(ops[last].flags & SOPF_SYNC)) ++last;
+    // lanes: leaf dots (first 32 lanes of a record), then the others
+    std::vector<CLane> leaf, rest;
+    std::vector<const SOp*> whole;
+    for (size_t k = first; k <= last; ++k) {
+      if (!fits_lanes(ops[k], lane_limit, dots)) {
+        whole.push_back(&ops[k]);
+        continue;
+      }
+      for (uint32_t c = 0; c < (1u << ops[k].rc); ++c)
+        ((ops[k].flags & SOPF_LEAFDOT) ? leaf : rest).push_back(make_lane(ops[k], c));
+    }
+    size_t nl = 0, nr = 0;
+    while (nl < leaf.size() || nr < rest.size()) {
+      Record r;
+      uint4 head{SOP_LANES, 0, 0, 0};
+      r.units.push_back(head);
+      for (uint32_t i = 0; i < max_lanes; ++i) {
+        CLane l{};
+        if (i < 32 && nl < leaf.size()) l = leaf[nl++];
+        else if (nr < rest.size()) l = rest[nr++];
+        else break;
+        r.units.push_back(unit_of(&l));
+      }
+      r.units[0].y = (uint32_t)r.units.size() - 1;
+      records.push_back(std::move(r));
+    }
+    for (const SOp* op : whole) {
+      Record r;
+      SOp plain = *op;
+      plain.flags &= (uint8_t)~SOPF_SYNC;
+      const unsigned char* p = reinterpret_cast<const unsigned char*>(&plain);
+      for (uint32_t u = 0; u < kSOpUnits; ++u) r.units.push_back(unit_of(p + 16 * u));
+      records.push_back(std::move(r));
+    }
+    records.back().level_end = true;
+    first = last + 1;
+  }
+  // batches; a level that ends with its batch needs no barrier of its own
+  std::vector<std::pair<size_t, size_t>> batches;
+  for (size_t i = 0; i < records.size();) {
+    size_t j = i;
+    uint32_t units = 1;
+    while (j < records.size() && units + records[j].units.size() <= half_units)
+      units += (uint32_t)records[j++].units.size();
+    batches.push_back({i, j});
+    i = j;
+  }
+  std::vector<uint32_t> sizes;
+  for (const auto& b : batches) {
+    uint32_t units = 1;
+    for (size_t k = b.first; k < b.second; ++k) units += (uint32_t)records[k].units.size();
+    sizes.push_back(units);
+  }
+  for (size_t n = 0; n < batches.size(); ++n) {
+    const auto& b = batches[n];
+    out.push_back(uint4{(uint32_t)(b.second - b.first), n + 1 < sizes.size() ? sizes[n + 1] : 0u,
+                        0, 0});
+    for (size_t k = b.first; k < b.second; ++k) {
+      if (records[k].level_end && k + 1 < b.second) records[k].units[0].x |= SOPF_SYNC << 24;
+      out.insert(out.end(), records[k].units.begin(), records[k].units.end());
+    }
+  }
+  return sizes[0];
+}
+
+void validate_cta_stream(const uint4* stream, size_t n, uint32_t units, uint32_t half_units,
+                         uint32_t table_elems, uint32_t arena_elems, int n_params) {
+  auto need = [&](bool ok, const char* what) {
+    if (!ok) fail(QTC_ERR_INVALID, "internal: task stream: %s", what);
+  };
+  const uint32_t team_elems = table_elems + arena_elems;
+  size_t at = 0;
+  while (units) {
+    need(units <= half_units && at + units <= n, "batch beyond the stage or the stream");
+    const uint32_t next = stream[at].y;
+    size_t u = at + 1;
+    for (uint32_t r = 0; r < stream[at].x; ++r) {
+      need(u < at + units, "records beyond their batch");
+      if ((stream[u].x & 15u) != SOP_LANES) {
+        u += kSOpUnits;   // (checked op by op before)
+        continue;
+      }
+      const uint32_t lanes = stream[u].y;
+      need(lanes >= 1 && u + 1 + lanes <= at + units, "lanes beyond their batch");
+      for (uint32_t i = 0; i < lanes; ++i) {
+        CLane l;
+        std::memcpy(&l, &stream[u + 1 + i], sizeof l);
+        const uint32_t ma = (uint32_t)(l.ya1 | l.ya2), mb = (uint32_t)(l.yb1 | l.yb2);
+        need((l.flags & 3) <= 2 && l.a + ma < team_elems && l.b + mb < team_elems, "lane operand");
+        // the two regions are addressed apart: an operand stays in its own
+        need((l.a < table_elems) == (l.a + ma < table_elems) &&
+                 (l.b < table_elems) == (l.b + mb < table_elems),
+             "lane operand across the table's end");
+        if (l.flags & CLF_STORE) need(l.out >= table_elems && l.out < team_elems, "lane output");
+        if (l.flags & CLF_DOT)
+          need(i < 32 && l.out < table_elems && l.slot < n_params && l.slot < kLaneDotSlots,
+               "lane leaf dot");
+      }
+      u += 1 + lanes;
+    }
+    need(u == at + units, "batch size");
+    at += units;
+    units = next;
+  }
+  need(at == n, "stream size");
 }
 
 }  // namespace qtc

@@ -3,6 +3,8 @@
 
 #include <stdint.h>
 
+#include <vector_types.h>
+
 #ifdef __CUDACC__
 #define QTC_HD __host__ __device__
 #else
@@ -89,7 +91,8 @@ enum SOpCode : uint8_t {
   SOP_CONTRACT = 0,    // out[c] = sum_y in1[.] * in2[.]  (Eq. 1, bit maps)
   SOP_LEAFGRAD = 1,    // grad[out] += sum_j in1[j] * in2[j], 2^rc terms
   SOP_RESULT = 2,      // network scalar = in1[0]
-  SOP_SEED = 3         // out[0] = 1 (adjoint of the root)
+  SOP_SEED = 3,        // out[0] = 1 (adjoint of the root)
+  SOP_LANES = 4        // stream record: small contractions, one output per thread
 };
 
 // Operand locations: by default an op offset is an element offset into the
@@ -113,6 +116,32 @@ enum SOpFlag : uint8_t {
 };
 constexpr int kLeafSlotByte = 15;     // (a leaf's output has at most 4 bits)
 constexpr uint32_t kNarrowMax = 128;  // outputs of a narrow op
+
+// A task's program is a stream of 16-byte units, read in batches that fit half
+// of the team's stage.  Batch: one unit (records, units of the next batch, 0, 0;
+// the last batch names 0 units), then its records.  Record: an SOp (5 units), or
+// a lanes record: a unit (SOP_LANES | flags << 24, lanes, 0, 0) and one CLane
+// per lane, which thread `lane` of the team runs.
+struct alignas(16) CLane {
+  uint16_t out;            // CLF_STORE: output; CLF_DOT: d(leaf)/dparam in the table
+  uint16_t a, b;           // first-term operands
+  uint8_t flags;           // bits 0-1: summed bits (0..2), CLaneFlag
+  uint8_t slot;            // CLF_DOT: parameter
+  uint16_t ya1, yb1;       // offsets of summed bit 0
+  uint16_t ya2, yb2;       // offsets of summed bit 1
+};
+enum CLaneFlag : uint8_t { CLF_STORE = 4, CLF_DOT = 8 };
+static_assert(sizeof(CLane) == 16, "one unit per lane");
+// Leaf dots of lanes go to an accumulator per (parameter, lane) of the warp that
+// owns the parameter (slot modulo the team's warps), summed at the task's end;
+// programs with more parameters keep their leaf dots in SOps.
+constexpr int kLaneDotSlots = 8;
+constexpr uint32_t kSOpUnits = 5;
+// Units of half of a stage of `bytes` bytes (at most 8 KiB a half).
+QTC_HD inline uint32_t smem_stage_half(uint32_t bytes) {
+  const uint32_t u = bytes / 32;
+  return u < 512 ? u : 512;
+}
 
 constexpr int kMaxSmemRank = 16;
 constexpr uint8_t kAbsent = 0xFF;
@@ -202,7 +231,8 @@ struct alignas(16) WStep {
 static_assert(sizeof(WStep) == 544, "WStep is staged as 34 16-byte words");
 
 struct TaskDev {
-  uint32_t op_begin, op_count;
+  uint32_t op_begin, op_count;     // warp teams: steps; CTA teams: first unit, units of the
+                                   // first batch
   uint32_t net;
   uint32_t arena_elems;
 };
@@ -225,12 +255,14 @@ struct ProgramDev {
   uint32_t table_elems;        // gate values + derivatives, in elements
   uint32_t table_bytes;        // table region, rounded to 16 bytes
   uint32_t team_bytes;         // per team: staged ops, then its arena
-  uint32_t stage_ops;          // ops staged per team at a time
+  uint32_t stage_ops;          // warp teams: steps staged per team at a time
+  uint32_t half_units;         // CTA teams: units of half the stage
+  int lane_dots;               // CTA teams: 1: lane accumulators of leaf dots
   uint32_t task_stride;        // warp teams: task t's steps start at t * task_stride
                                // (0: at tasks[t].op_begin)
   const TaskDev* tasks;
   int n_tasks;
-  const SOp* ops;              // CTA teams
+  const uint4* stream;         // CTA teams: programs
   const WStep* wsteps;         // warp teams
   int n_params;
   int n_nets;
@@ -381,13 +413,13 @@ enum GTaskKind : uint8_t { GT_SMEM = 0, GT_CHUNK = 1, GT_TC = 2 };
 struct GTask {
   uint8_t kind;
   uint8_t pad[3];
-  uint32_t a;              // SMEM: first op; CHUNK, TC: step index
-  uint32_t b;              // SMEM: op count; CHUNK: chunk index; TC: tile index
+  uint32_t a;              // SMEM: first unit; CHUNK, TC: step index
+  uint32_t b;              // SMEM: units of the first batch; CHUNK: chunk index; TC: tile index
   uint32_t net;
   uint32_t wait_begin;     // into the wait list
   uint32_t wait_count;
   uint32_t signal;         // SMEM: counter incremented when done (~0u: none)
-  uint32_t pad2;
+  uint32_t arena_elems;    // SMEM: elements of its arena (the stage follows it)
 };
 
 struct WaitDev {
@@ -412,11 +444,11 @@ struct GraphProgDev {
   int n_gates;
   uint32_t table_elems;
   uint32_t table_bytes;        // gate table region, 16-byte rounded
-  uint32_t arena_bytes;        // shared-memory arena of SMEM tasks
-  uint32_t stage_ops;          // ops staged at a time
+  uint32_t arena_bytes;        // work region of a team
+  int lane_dots;               // 1: SMEM tasks keep lane accumulators of leaf dots
   const GTask* tasks;
   int n_tasks;
-  const SOp* ops;
+  const uint4* stream;         // programs of SMEM tasks
   const GStep* steps;
   const TStep* tsteps;         // tensor-core GEMMs
   const WaitDev* waits;

@@ -414,9 +414,8 @@ __device__ __forceinline__ void sum_outputs(const SOp& op, const T* a, const T* 
 // value and the operands' loads.  Sums run in order of the summed index.  Bound
 // by latency: programs are chains of levels of a few small ops.  Against one
 // barrier per op with the maps walked bit by bit for every operand element, the
-// p=2 n=100 gradient step on CTA teams went from 520 to 280 us, the dense one's
-// graph launch from 1.83 to 1.47 ms, complex128 n=20 full networks from 4.30 to
-// 3.89 ms.
+// p=2 n=100 gradient launch on CTA teams went from 495 to 209 us, the dense
+// one's graph launch from 1.83 to 1.47 ms.
 template <typename T, int kLog>
 __device__ __noinline__ void contract_by(const SOp& op, T* out, const T* a, const T* b,
                                          uint32_t t) {
@@ -545,6 +544,104 @@ __device__ __forceinline__ void run_op(const SOp& op, const TeamT& team, const A
     }
   }
   if (flags & SOPF_SYNC) team.sync();
+}
+
+// A team's program (see CLane): runs the stream's batches, each copied into one
+// half of `stage` while the other half's records run.  `lacc`: accumulators of
+// lane leaf dots (n_dots parameters x 32 lanes), or null.  Every record of a
+// level ends in the same barrier; the next record's header and this thread's
+// lane are read before it, so a level of lanes costs about one round trip
+// through shared memory and the barrier (an op run from its record forms its
+// offsets first, 100 instructions or so).  The p=2 n=100 gradient launch (250
+// networks of about 485 ops in 163 levels): 209 -> 115 us.
+template <typename T, int kLog, typename TeamT, typename At, typename G, typename Result>
+__device__ __forceinline__ void run_stream(const uint4* src, uint32_t units, uint4* stage,
+                                           uint32_t half, const TeamT& team, const At& at,
+                                           T* table, T* lacc, int n_dots, G* grad,
+                                           const Result& result) {
+  const uint32_t tid = team.tid, lane = tid & 31u, warp = tid >> 5;
+  constexpr uint32_t kWarps = 1u << (kLog - 5);
+  if (lacc)
+    for (int q = (int)warp; q < n_dots; q += (int)kWarps) lacc[q * 32 + lane] = czero<T>();
+  for (uint32_t u = tid; u < units; u += 1u << kLog) cp_async16(stage + u, src + u);
+  uint4* cur = stage;
+  uint4* other = stage + half;
+  while (units) {
+    cp_async_wait_all();
+    team.sync();
+    const uint4 batch = cur[0];
+    src += units;
+    for (uint32_t u = tid; u < batch.y; u += 1u << kLog) cp_async16(other + u, src + u);
+    const uint4* rec = cur + 1;
+    const uint4* end = cur + units;
+    uint4 head = rec[0], L = make_uint4(0, 0, 0, 0);
+    bool have = (head.x & 15u) == SOP_LANES && tid < head.y;
+    if (have) L = rec[1 + tid];
+    while (rec < end) {
+      if ((head.x & 15u) != SOP_LANES) {
+        run_op<T, kLog>(*reinterpret_cast<const SOp*>(rec), team, at, (const T*)table, grad, result);
+        rec += kSOpUnits;
+        if (rec < end) {
+          head = rec[0];
+          have = (head.x & 15u) == SOP_LANES && tid < head.y;
+          if (have) L = rec[1 + tid];
+        }
+        continue;
+      }
+      const uint32_t n = head.y;
+      const bool sync = (head.x >> 24) & SOPF_SYNC;
+      const uint4* next = rec + 1 + n;
+      for (uint32_t i = tid;;) {
+        if (have) {
+          const uint32_t flags = (L.y >> 16) & 0xffu;
+          const T* a = at(L.x >> 16, 0u);
+          const T* b = at(L.y & 0xffffu, 0u);
+          const uint32_t ya1 = L.z & 0xffffu, yb1 = L.z >> 16;
+          const uint32_t ya2 = L.w & 0xffffu, yb2 = L.w >> 16;
+          const T a0 = a[0], b0 = b[0], a1 = a[ya1], b1 = b[yb1];
+          T acc = cfma(a0, b0, czero<T>());
+          if (flags & 3u) acc = cfma(a1, b1, acc);
+          if (flags & 2u) {
+            const T a2 = a[ya2], b2 = b[yb2], a3 = a[ya1 | ya2], b3 = b[yb1 | yb2];
+            acc = cfma(a2, b2, acc);
+            acc = cfma(a3, b3, acc);
+          }
+          if (flags & CLF_STORE) *at(L.x & 0xffffu, 0u) = acc;
+          if (flags & CLF_DOT) {
+            T* s = lacc + (L.y >> 24) * 32u + lane;
+            *s = cfma(acc, table[L.x & 0xffffu], *s);
+          }
+        }
+        i += 1u << kLog;
+        if ((i & ~31u) >= n) break;   // (uniform in a warp)
+        have = i < n;
+        if (have) L = rec[1 + i];
+      }
+      rec = next;
+      have = false;
+      if (rec < end) {
+        head = rec[0];
+        have = (head.x & 15u) == SOP_LANES && tid < head.y;
+        if (have) L = rec[1 + tid];
+      }
+      if (sync) team.sync();
+    }
+    units = batch.y;
+    uint4* t = cur;
+    cur = other;
+    other = t;
+  }
+  team.sync();
+  if (lacc) {
+    for (int q = (int)warp; q < n_dots; q += (int)kWarps) {
+      const T v = warp_csum(lacc[q * 32 + lane], 32u);
+      if (lane == 0) {
+        grad[2 * q] += (G)v.x;
+        grad[2 * q + 1] += (G)v.y;
+      }
+    }
+    team.sync();
+  }
 }
 
 }  // namespace qtc

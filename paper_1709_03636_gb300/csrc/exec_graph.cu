@@ -126,29 +126,24 @@ __device__ __noinline__ void run_smem_task(const GraphProgDev& prog, const GTask
   const int P = prog.n_params;
   const int stride = 2 + 2 * P;
   for (int i = team.tid; i < 2 * P; i += team.size) s_grad[i] = 0.0;
-  SOp* stage = reinterpret_cast<SOp*>(work);
-  T* arena = reinterpret_cast<T*>(work + (size_t)prog.stage_ops * sizeof(SOp));
+  // [lane accumulators | arena | stage (two halves)]
   T* gbase = reinterpret_cast<T*>(prog.gbase);
-  constexpr int kWords = sizeof(SOp) / sizeof(uint4);
-  for (uint32_t base = 0; base < task.b; base += prog.stage_ops) {
-    const uint32_t n = min(prog.stage_ops, task.b - base);
-    team.sync();
-    const uint4* src = reinterpret_cast<const uint4*>(prog.ops + task.a + base);
-    uint4* dst = reinterpret_cast<uint4*>(stage);
-    for (uint32_t w = team.tid; w < n * kWords; w += team.size) dst[w] = src[w];
-    team.sync();
-    for (uint32_t k = 0; k < n; ++k)
-      run_op<T, kGraphBlockLog>(
-          stage[k], team,
-          [&](uint32_t off, uint32_t global) {
-            return locate(off, global != 0, gbase, table, arena, prog.table_elems);
-          },
-          table, s_grad, [&](T r) {
-            const double2 v = to_d2(r);
-            prog.results[(size_t)task.net * stride] = v.x;
-            prog.results[(size_t)task.net * stride + 1] = v.y;
-          });
-  }
+  const bool dots = prog.lane_dots != 0;
+  T* lacc = dots ? reinterpret_cast<T*>(work) : nullptr;
+  T* arena = reinterpret_cast<T*>(work) + (dots ? 32 * P : 0);
+  uint4* stage = reinterpret_cast<uint4*>(arena + task.arena_elems);
+  const uint32_t half = smem_stage_half((uint32_t)(work + prog.arena_bytes -
+                                                   reinterpret_cast<unsigned char*>(stage)));
+  run_stream<T, kGraphBlockLog>(
+      prog.stream + task.a, task.b, stage, half, team,
+      [&](uint32_t off, uint32_t global) {
+        return locate(off, global != 0, gbase, table, arena, prog.table_elems);
+      },
+      table, lacc, P, s_grad, [&](T r) {
+        const double2 v = to_d2(r);
+        prog.results[(size_t)task.net * stride] = v.x;
+        prog.results[(size_t)task.net * stride + 1] = v.y;
+      });
   for (int i = team.tid; i < 2 * P; i += team.size)
     if (s_grad[i] != 0.0) atomicAdd(&prog.results[(size_t)task.net * stride + 2 + i], s_grad[i]);
   signal_done(prog, task.signal, team);

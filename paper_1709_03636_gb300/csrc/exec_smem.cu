@@ -284,21 +284,22 @@ __global__ void __maxnreg__(kExecMaxRegs) smem_exec_kernel(const ProgramDev prog
   // A CTA team reads the gate table at the start of shared memory; a warp
   // team keeps its own copy between its staged steps and its arena, so its
   // table and arena offsets run on from one another.
-  using OpT = typename std::conditional<kWarp, WStep, SOp>::type;
   const Team<kWarp> team;
   const int P = prog.n_params;
   const int teams_per_cta = blockDim.x / team.size;
   unsigned char* team_base = smem_raw + prog.table_bytes + (size_t)team.id * prog.team_bytes;
-  OpT* stage = reinterpret_cast<OpT*>(team_base);
-  T* after_stage = reinterpret_cast<T*>(team_base + (size_t)prog.stage_ops * sizeof(OpT));
-  const bool lane_grad = kWarp && prog.want_grad && P <= kWarpLaneGradSlots;
+  WStep* stage = reinterpret_cast<WStep*>(team_base);
+  // (CTA teams: the table, then [stage | lane accumulators | arena])
+  T* after_stage = reinterpret_cast<T*>(
+      team_base + (kWarp ? (size_t)prog.stage_ops * sizeof(WStep) : (size_t)prog.half_units * 32));
+  const bool lane_grad =
+      kWarp ? prog.want_grad && P <= kWarpLaneGradSlots : prog.lane_dots != 0;
   T* table = kWarp ? after_stage + (lane_grad ? 32 * P : 0) : reinterpret_cast<T*>(smem_raw);
-  T* arena = kWarp ? table + prog.table_elems : after_stage;
-  const OpT* ops = kWarp ? reinterpret_cast<const OpT*>(prog.wsteps)
-                         : reinterpret_cast<const OpT*>(prog.ops);
+  T* arena = kWarp ? table + prog.table_elems : after_stage + (lane_grad ? 32 * P : 0);
+  const WStep* ops = prog.wsteps;
   R* grad = s_grad[team.id];
   const int stride = 2 + 2 * P;
-  constexpr int kWords = sizeof(OpT) / sizeof(uint4);
+  constexpr int kWords = sizeof(WStep) / sizeof(uint4);
   const uint32_t stage_s = smem_u32(stage), table_s = smem_u32(table);
   const uint32_t lacc_s = smem_u32(after_stage) + team.tid * (uint32_t)sizeof(T);
   const uint32_t res_s = smem_u32(&s_res[team.id]);
@@ -328,7 +329,9 @@ __global__ void __maxnreg__(kExecMaxRegs) smem_exec_kernel(const ProgramDev prog
     task = prog.tasks[t];
   } else if (t < (unsigned)prog.n_tasks) {
     uint4* dst = reinterpret_cast<uint4*>(stage);
-    if (kWarp && prog.task_stride) {
+    if (!kWarp) {
+      task = prog.tasks[t];
+    } else if (prog.task_stride) {
       // fixed stride: the copy starts before the task record arrives
       const uint4* src = reinterpret_cast<const uint4*>(ops + (size_t)t * prog.task_stride);
       for (uint32_t w = team.tid; w < prog.stage_ops * kWords; w += team.size)
@@ -352,7 +355,7 @@ __global__ void __maxnreg__(kExecMaxRegs) smem_exec_kernel(const ProgramDev prog
   while (t < (unsigned)prog.n_tasks) {
     const double w_net = prog.weights[task.net];  // used once the network is done
     for (int i = team.tid; i < 2 * P; i += team.size) grad[i] = R(0);
-    if (lane_grad)
+    if (kWarp && lane_grad)
       for (int q = 0; q < P; ++q) sts_c(lacc_s + q * 32u * (uint32_t)sizeof(T), czero<T>());
     if constexpr (kStream) {
       const WStep* gs = prog.wsteps + task.op_begin;
@@ -401,28 +404,35 @@ __global__ void __maxnreg__(kExecMaxRegs) smem_exec_kernel(const ProgramDev prog
         team.sync();
       }
     }
-    for (uint32_t base = 0; !kStream && base < task.op_count; base += prog.stage_ops) {
-      const uint32_t n = min(prog.stage_ops, task.op_count - base);
-      if (!staged) {
-        // stage a chunk of the op list with one cooperative copy
+    if constexpr (!kWarp) {
+      team.sync();   // the slots are cleared
+      run_stream<T, kExecBlockLog>(
+          prog.stream + task.op_begin, task.op_count, reinterpret_cast<uint4*>(stage),
+          prog.half_units, team,
+          [&](uint32_t off, uint32_t) { return resolve(off, table, arena, prog.table_elems); },
+          table, lane_grad ? after_stage : nullptr, P, grad,
+          [&](T v) { s_res[team.id] = to_d2(v); });
+    }
+    if constexpr (kWarp && !kStream) {
+      for (uint32_t base = 0; base < task.op_count; base += prog.stage_ops) {
+        const uint32_t n = min(prog.stage_ops, task.op_count - base);
+        if (!staged) {
+          // stage a chunk of the op list with one cooperative copy
+          team.sync();
+          const uint4* src = reinterpret_cast<const uint4*>(ops + task.op_begin + base);
+          uint4* dst = reinterpret_cast<uint4*>(stage);
+          for (uint32_t w = team.tid; w < n * kWords; w += team.size) dst[w] = src[w];
+        }
+        staged = false;
         team.sync();
-        const uint4* src = reinterpret_cast<const uint4*>(ops + task.op_begin + base);
-        uint4* dst = reinterpret_cast<uint4*>(stage);
-        for (uint32_t w = team.tid; w < n * kWords; w += team.size) dst[w] = src[w];
-      }
-      staged = false;
-      team.sync();
-      // warp programs: the next step's header and this lane's descriptor are
-      // loaded while the current step runs
-      uint32_t h_next = 0;
-      uint4 l_next = make_uint4(0, 0, 0, 0);
-      if (kWarp) {
+        // warp programs: the next step's header and this lane's descriptor are
+        // loaded while the current step runs
+        uint32_t h_next = 0;
+        uint4 l_next = make_uint4(0, 0, 0, 0);
         h_next = lds_u32(stage_s);
         l_next = lds_u4(stage_s + 16 + 16 * team.tid);
-      }
-      for (uint32_t k = 0; k < n; ++k) {
-        const OpT& op = stage[k];
-        if constexpr (kWarp) {
+        for (uint32_t k = 0; k < n; ++k) {
+          const WStep& op = stage[k];
           const uint32_t h = h_next;  // solo | rounds << 8
           const uint4 L = l_next;
           if (k + 1 < n) {
@@ -452,16 +462,11 @@ __global__ void __maxnreg__(kExecMaxRegs) smem_exec_kernel(const ProgramDev prog
               if (team.tid == 0) *out = from_d2<T>(make_double2(1.0, 0.0));
             }
           }
-        } else {
-          run_op<T, kExecBlockLog>(
-              op, team,
-              [&](uint32_t off, uint32_t) { return resolve(off, table, arena, prog.table_elems); },
-              table, grad, [&](T v) { s_res[team.id] = to_d2(v); });
+          team.sync();
         }
-        if (kWarp) team.sync();
       }
     }
-    if (lane_grad) {
+    if (kWarp && lane_grad) {
       // sum the lanes' accumulators into the network's slots
       for (int q = 0; q < P; ++q) {
         T v = warp_csum(lds_c<T>(lacc_s + q * 32u * (uint32_t)sizeof(T)), 32u);

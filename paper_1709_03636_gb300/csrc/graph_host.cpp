@@ -51,7 +51,7 @@ double task_time_estimate(const GUnit& u, size_t elem, int teams) {
 }
 
 WaveHost assemble_wave(const std::vector<int>& nets, const std::vector<NetGraph>& graphs,
-                       size_t elem, int teams) {
+                       size_t elem, int teams, const HostProgram& hp) {
   WaveHost w;
   std::vector<std::vector<uint32_t>> ctr(nets.size()), arrive(nets.size());
   std::vector<uint64_t> base(nets.size());
@@ -101,15 +101,24 @@ WaveHost assemble_wave(const std::vector<int>& nets, const std::vector<NetGraph>
     t.signal = 0xFFFFFFFFu;
     if (u.kind == GT_SMEM) {
       t.kind = GT_SMEM;
-      t.a = (uint32_t)w.ops.size();
-      t.b = (uint32_t)u.ops.size();
       t.signal = ctr[k][ui];
-      for (SOp op : u.ops) {
+      std::vector<SOp> ops = u.ops;
+      for (SOp& op : ops) {
         if (op.flags & SOPF_OUT_GLOBAL) op.out = rebase32(base[k], op.out);
         if (op.flags & SOPF_IN1_GLOBAL) op.in1 = rebase32(base[k], op.in1);
         if (op.flags & SOPF_IN2_GLOBAL) op.in2 = rebase32(base[k], op.in2);
-        w.ops.push_back(op);
       }
+      validate_cta_ops(ops.data(), ops.size(), hp.table_elems, u.arena_elems, gsize, hp.n_params,
+                       kGraphWarps);
+      const bool dots = hp.lane_dots;
+      const uint32_t half = smem_stage_half(
+          hp.work_bytes - (uint32_t)(((dots ? 32u * (uint32_t)hp.n_params : 0u) + u.arena_elems) *
+                                     elem));
+      t.arena_elems = u.arena_elems;
+      t.a = (uint32_t)w.stream.size();
+      t.b = build_cta_stream(ops, half, kLaneLimit, dots, w.stream);
+      validate_cta_stream(w.stream.data() + t.a, w.stream.size() - t.a, t.b, half, hp.table_elems,
+                          u.arena_elems, hp.n_params);
     } else if (u.kind == GT_TC) {
       TStep ts = u.tstep;
       ts.net = (uint32_t)nets[k];
@@ -223,7 +232,7 @@ uint64_t runs_offset_host(const GRuns& r, uint64_t idx) {
 // against the dependencies, so that a lowering mistake is an error on the
 // host instead of a bad address or a wait that never ends on the device.
 void validate_wave(const WaveHost& w, uint32_t table_elems, uint32_t arena_elems,
-                   size_t elem_of_wave, size_t work_bytes, int n_params) {
+                   size_t elem_of_wave, size_t work_bytes) {
   auto check_ref = [&](uint32_t off, bool global, uint64_t max_index, const char* what) {
     const uint64_t end = (uint64_t)off + max_index + 1;
     if (global) {
@@ -238,11 +247,9 @@ void validate_wave(const WaveHost& w, uint32_t table_elems, uint32_t arena_elems
     if (t.wait_begin + t.wait_count > w.waits.size())
       fail(QTC_ERR_INVALID, "internal: wait list out of range");
     if (t.kind == GT_SMEM) {
-      if ((uint64_t)t.a + t.b > w.ops.size()) fail(QTC_ERR_INVALID, "internal: op range");
+      if ((uint64_t)t.a + t.b > w.stream.size()) fail(QTC_ERR_INVALID, "internal: stream range");
       if (t.signal != 0xFFFFFFFFu && t.signal >= w.n_counters)
         fail(QTC_ERR_INVALID, "internal: signal counter out of range");
-      validate_cta_ops(w.ops.data() + t.a, t.b, table_elems, arena_elems, w.global_elems, n_params,
-                       kGraphWarps);
     } else if (t.kind == GT_TC) {
       if (t.a >= w.tsteps.size()) fail(QTC_ERR_INVALID, "internal: GEMM index");
       const TStep& ts = w.tsteps[t.a];
@@ -550,34 +557,36 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
   uint32_t max_arena = 0;
   for (const NetGraph& g : graphs)
     for (const GUnit& u : g.units) max_arena = std::max(max_arena, u.arena_elems);
-  hp.tensor_cores = false;
-  for (auto& wnets : waves) {
-    std::sort(wnets.begin(), wnets.end());
-    hp.waves.push_back(assemble_wave(wnets, graphs, elem, opts.sm_count * 4));
-
-    if (!hp.waves.back().tsteps.empty()) hp.tensor_cores = true;
-    hp.max_global_elems = std::max(hp.max_global_elems, hp.waves.back().global_elems);
-    hp.max_counters = std::max(hp.max_counters, hp.waves.back().n_counters);
-  }
   hp.max_arena = max_arena;
-  hp.stage_ops = 32;
   auto round16 = [](size_t x) { return (uint32_t)((x + 15) & ~size_t(15)); };
-  const size_t smem_task = (size_t)hp.stage_ops * sizeof(SOp) + (size_t)max_arena * elem;
+  // a subtree task keeps at least 2560 bytes beside the largest arena for its
+  // lane accumulators and its stage (other tasks stage more)
+  const size_t smem_task = 2560 + (size_t)max_arena * elem;
   const size_t chunk_task = 2 * (size_t)kYTab * sizeof(uint32_t) + 256 * elem +
                             3 * (size_t)kMaxChunkRows * sizeof(uint32_t);
   size_t tile_task = 0;
   hp.tiles = false;
-  for (const WaveHost& w : hp.waves)
-    for (const GStep& st : w.steps)
-      if (st.flags & GSF_TILE) {
-        tile_task = std::max(tile_task, tile_region_bytes(st, elem));
+  hp.tensor_cores = false;
+  for (const NetGraph& g : graphs)
+    for (const GUnit& u : g.units) {
+      if (u.kind == GT_TC) hp.tensor_cores = true;
+      if (u.kind == GT_CHUNK && (u.step.flags & GSF_TILE)) {
+        tile_task = std::max(tile_task, tile_region_bytes(u.step, elem));
         hp.tiles = true;
       }
+    }
+  hp.lane_dots = hp.want_grad && hp.n_params <= kLaneDotSlots &&
+                 32 * hp.n_params * elem <= 2560 - 512;
   hp.work_bytes = round16(std::max({smem_task, chunk_task, tile_task}));
   hp.table_bytes = round16((size_t)hp.table_elems * elem);
   hp.smem = hp.table_bytes + (size_t)(hp.tensor_cores ? 4 : 1) * hp.work_bytes;
-  for (const WaveHost& w : hp.waves) 
-    validate_wave(w, hp.table_elems, max_arena, elem, hp.work_bytes, hp.n_params);
+  for (auto& wnets : waves) {
+    std::sort(wnets.begin(), wnets.end());
+    hp.waves.push_back(assemble_wave(wnets, graphs, elem, opts.sm_count * 4, hp));
+    hp.max_global_elems = std::max(hp.max_global_elems, hp.waves.back().global_elems);
+    hp.max_counters = std::max(hp.max_counters, hp.waves.back().n_counters);
+  }
+  for (const WaveHost& w : hp.waves) validate_wave(w, hp.table_elems, max_arena, elem, hp.work_bytes);
   if (hp.smem > max_dynamic)
     fail(QTC_ERR_UNSUPPORTED, "graph program needs %zu bytes of shared memory (limit %zu)",
          hp.smem, max_dynamic);

@@ -190,6 +190,18 @@ void schedule_cta_ops(std::vector<SOp>& ops, uint32_t table_elems, int n_warps);
 void validate_cta_ops(const SOp* ops, size_t n, uint32_t table_elems, uint32_t arena_elems,
                       uint64_t global_elems, int n_params, int n_warps);
 
+// Appends a task's scheduled ops as a stream (see CLane) for a stage of twice
+// half_units units; ops of at most lane_limit outputs become lanes, leaf dots
+// among them only with `dots`.  Returns the units of the first batch.
+uint32_t build_cta_stream(const std::vector<SOp>& ops, uint32_t half_units, uint32_t lane_limit,
+                          bool dots, std::vector<uint4>& out);
+// Host check of one task's stream (its ops already checked).
+void validate_cta_stream(const uint4* stream, size_t n, uint32_t units, uint32_t half_units,
+                         uint32_t table_elems, uint32_t arena_elems, int n_params);
+// Outputs of an op that becomes lanes: up to 16 of them cost no more memory than
+// its record, on average; 4 never more (used where memory is short).
+constexpr uint32_t kLaneLimit = 16, kLaneLimitSmall = 4;
+
 // Lowers one plan to a shared-memory op program.  table_elems: size of the
 // gate value + derivative region that precedes the arena.  Intermediates and
 // adjoints of at most private_below elements keep arena buffers of their own
@@ -313,7 +325,7 @@ struct ProgramOptions {
 // work-buffer size and dependency counters.
 struct WaveHost {
   std::vector<GTask> tasks;
-  std::vector<SOp> ops;
+  std::vector<uint4> stream;       // programs of SMEM tasks
   std::vector<GStep> steps;
   std::vector<TStep> tsteps;
   std::vector<WaitDev> waits;
@@ -330,14 +342,17 @@ struct HostProgram {
   size_t max_dynamic = 0;          // shared-memory budget it was lowered for
   std::vector<GateEntryDev> gates;
   std::vector<TaskDev> tasks;
-  std::vector<SOp> ops;            // CTA teams (empty for warp teams)
+  std::vector<SOp> ops;            // CTA teams (empty for warp teams): what `stream` holds
+  std::vector<uint4> stream;       // CTA teams: programs
   std::vector<WStep> wsteps;       // warp teams
   std::vector<uint8_t> coef;       // warp teams: gate table coefficient records
   std::vector<double> weights;
   uint32_t table_elems = 0, max_arena = 0;
   uint32_t table_bytes = 0;        // gate table region, 16-byte rounded
   uint32_t team_bytes = 0;         // per team: staged ops + arena
-  uint32_t stage_ops = 0;          // ops staged per team at a time
+  uint32_t stage_ops = 0;          // warp teams: steps staged per team at a time
+  uint32_t half_units = 0;         // CTA teams: units of half the stage
+  bool lane_dots = false;          // CTA teams, graph form: lane accumulators of leaf dots
   uint32_t task_stride = 0;        // warp steps of task t start at t * task_stride (0: packed)
   bool warp_teams = false;         // one network per warp (small networks)
   bool stream_steps = false;       // warp teams read their steps from global memory

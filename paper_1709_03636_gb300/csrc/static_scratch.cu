@@ -81,7 +81,7 @@ extern "C" qtc_status qtc_qaoa_expectation_static(qtc_batch* b, const double* pa
     const size_t o_gates = 0;
     const size_t o_tasks = align256(o_gates + sizeof(GateEntryDev) * G);
     const size_t o_ops = align256(o_tasks + sizeof(TaskDev) * hp.tasks.size());
-    const size_t o_wsteps = align256(o_ops + sizeof(SOp) * hp.ops.size());
+    const size_t o_wsteps = align256(o_ops + sizeof(uint4) * hp.stream.size());
     const size_t o_coef = align256(o_wsteps + sizeof(WStep) * hp.wsteps.size());
     const size_t o_weights = align256(o_coef + hp.coef.size());
     const size_t o_results = align256(o_weights + sizeof(double) * N);
@@ -103,9 +103,10 @@ extern "C" qtc_status qtc_qaoa_expectation_static(qtc_batch* b, const double* pa
       cuda_check(cudaMemcpyAsync(base + o_tasks, hp.tasks.data(),
                                  sizeof(TaskDev) * hp.tasks.size(), cudaMemcpyHostToDevice, s),
                  "upload tasks");
-      if (!hp.ops.empty())
-        cuda_check(cudaMemcpyAsync(base + o_ops, hp.ops.data(), sizeof(SOp) * hp.ops.size(),
-                                   cudaMemcpyHostToDevice, s), "upload ops");
+      if (!hp.stream.empty())
+        cuda_check(cudaMemcpyAsync(base + o_ops, hp.stream.data(),
+                                   sizeof(uint4) * hp.stream.size(), cudaMemcpyHostToDevice, s),
+                   "upload programs");
       if (!hp.wsteps.empty())
         cuda_check(cudaMemcpyAsync(base + o_wsteps, hp.wsteps.data(),
                                    sizeof(WStep) * hp.wsteps.size(),
@@ -135,11 +136,13 @@ extern "C" qtc_status qtc_qaoa_expectation_static(qtc_batch* b, const double* pa
     d.table_bytes = hp.table_bytes;
     d.team_bytes = hp.team_bytes;
     d.stage_ops = hp.stage_ops;
+    d.half_units = hp.half_units;
+    d.lane_dots = hp.lane_dots;
     d.task_stride = hp.task_stride;
     d.coef = base + o_coef;
     d.tasks = (const TaskDev*)(base + o_tasks);
     d.n_tasks = (int)hp.tasks.size();
-    d.ops = (const SOp*)(base + o_ops);
+    d.stream = (const uint4*)(base + o_ops);
     d.wsteps = (const WStep*)(base + o_wsteps);
     d.n_params = P;
     d.n_nets = N;
