@@ -294,6 +294,9 @@ extern "C" qtc_status qtc_selftest_tile_steps(qtc_batch* b, int dtype, int want_
         if ((st.flags & GSF_TILE) && st.rc + st.ry <= max_bits) {
           err = std::max(err, emulate_tile_step(st, seed++));
           ++n;
+        } else if ((st.flags & GSF_STAGE) && st.rc + st.ry <= max_bits) {
+          err = std::max(err, emulate_stage_step(st, seed++));
+          ++n;
         } else if ((st.flags & GSF_ROWS) && st.rc + st.ry <= max_bits) {
           err = std::max(err, emulate_rows_step(st, seed++));
           ++n;

@@ -79,7 +79,7 @@ double op_cycles(const SOp& op) {
 
 }  // namespace
 
-void schedule_cta_ops(std::vector<SOp>& ops, uint32_t table_elems, int n_warps) {
+double schedule_cta_ops(std::vector<SOp>& ops, uint32_t table_elems, int n_warps) {
   // leaf dots into the adjoints that produce their operand (nothing else
   // reads a leaf's adjoint)
   std::vector<SOp> in;
@@ -152,6 +152,7 @@ void schedule_cta_ops(std::vector<SOp>& ops, uint32_t table_elems, int n_warps) 
   for (int i = 0; i < n; ++i) by_level[level[i]].push_back(i);
   ops.clear();
   std::vector<double> load(n_warps);
+  double cycles = 0;
   for (auto& members : by_level) {
     // narrow ops first, longest first, each to the warp with the least to do
     // (leaf dots to the first warp, so that the order of their terms is fixed);
@@ -162,8 +163,10 @@ void schedule_cta_ops(std::vector<SOp>& ops, uint32_t table_elems, int n_warps) 
       return nx && op_cycles(in[x]) > op_cycles(in[y]);
     });
     std::fill(load.begin(), load.end(), 0.0);
+    cycles += 200;
     for (int i : members) {
       SOp op = in[i];
+      if (!(op.flags & SOPF_NARROW)) cycles += op_cycles(op);
       if (op.flags & SOPF_NARROW) {
         int w = (int)(std::min_element(load.begin(), load.end()) - load.begin());
         if (op.code == SOP_LEAFGRAD || (op.flags & SOPF_LEAFDOT)) w = 0;
@@ -173,7 +176,9 @@ void schedule_cta_ops(std::vector<SOp>& ops, uint32_t table_elems, int n_warps) 
       ops.push_back(op);
     }
     if (!members.empty()) ops.back().flags |= SOPF_SYNC;
+    cycles += *std::max_element(load.begin(), load.end());
   }
+  return cycles;
 }
 
 void validate_cta_ops(const SOp* ops, size_t n, uint32_t table_elems, uint32_t arena_elems,

@@ -308,9 +308,31 @@ enum GStepFlag : uint16_t {
                        //   complex64 terms are read as 16-byte element pairs
   GSF_LANES_Y = 64,    // split: the summed index's low bits are A's (or B's) lowest
                        //   bits, so a warp's lanes run over it (one warp per output)
-  GSF_ROWS = 128       // rows taken four at a time in the order of `rows`, so that the
+  GSF_ROWS = 128,      // rows taken four at a time in the order of `rows`, so that the
                        //   four share operand elements (`share`): fewer loads per term
+  GSF_SUM8 = 256,      // sums over rows in eight accumulators (value y to y modulo 8),
+                       //   folded every kYTab values
+  GSF_STAGE = 512,     // 2^share outputs per task, their operands' footprints copied through
+                       //   shared memory in batches of summed values
+  GSF_SUM_PAIR4 = 1024 // GSF_STAGE: four accumulators of adjacent pairs (pair p to p modulo 4)
 };
+
+// GSF_STAGE: a row's footprint in an operand is one element per value of the
+// low output bits that the operand holds.  A task's work region holds the
+// offsets of both footprints, two batches of summed-index offsets and two of
+// the footprints' elements.
+constexpr uint32_t kStageOffsets = 2 * 256 * sizeof(uint32_t);
+constexpr uint32_t kStageMaxY = 256;                     // summed values per batch
+constexpr uint32_t kStageHead = kStageOffsets + 2 * kStageMaxY * 2 * sizeof(uint32_t);
+constexpr uint32_t kStageBytes = 32768;                  // of the work region
+// log2 of the summed values of a batch (0: fewer than 16 fit, not staged)
+QTC_HD inline int stage_log2_y(uint32_t footprint_elems, uint32_t elem_bytes, int ry) {
+  int l = 0;
+  while (l < 8 && l < ry &&
+         2ull * (2u << l) * footprint_elems * elem_bytes <= kStageBytes - kStageHead)
+    ++l;
+  return l >= 4 ? l : 0;
+}
 
 // How the four rows of a GSF_ROWS group share operands: row-counter bit 0 and
 // bit 1 map to output labels missing from A (A's element is the same for both
@@ -380,7 +402,8 @@ struct alignas(16) GStep {
   uint32_t net;
   uint16_t flags;
   int16_t slot;             // leafgrad: parameter slot
-  uint8_t rc, ry, share, pad1;  // share: GRowShare of a GSF_ROWS step
+  uint8_t rc, ry, share;    // share: GRowShare of a GSF_ROWS step; GSF_STAGE: log2 outputs
+  uint8_t stage_y;          // GSF_STAGE: log2 of the summed values per batch
   GRuns ca, cb;             // output bits -> A bits, B bits
   GRuns ya, yb;             // summed bits -> A bits, B bits
   GRuns rows;               // GSF_ROWS: row counter bits -> output row bits

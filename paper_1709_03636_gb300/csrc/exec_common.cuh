@@ -417,7 +417,7 @@ __device__ __forceinline__ void sum_outputs(const SOp& op, const T* a, const T* 
 // p=2 n=100 gradient launch on CTA teams went from 495 to 209 us, the dense
 // one's graph launch from 1.83 to 1.47 ms.
 template <typename T, int kLog>
-__device__ __noinline__ void contract_by(const SOp& op, T* out, const T* a, const T* b,
+__device__ __forceinline__ void contract_by(const SOp& op, T* out, const T* a, const T* b,
                                          uint32_t t) {
   const uint32_t nout = 1u << op.rc, lane = t & 31u;
   if ((t & ~31u) >= nout) return;   // whole warps
@@ -466,7 +466,7 @@ __device__ __noinline__ void contract_by(const SOp& op, T* out, const T* a, cons
 // derivative `der` goes to the gradient slot (one warp owns a slot, so the order
 // of its terms is fixed).
 template <typename T, typename G>
-__device__ __noinline__ void adjoint_by_warp(const SOp& op, T* out, const T* a, const T* b,
+__device__ __forceinline__ void adjoint_by_warp(const SOp& op, T* out, const T* a, const T* b,
                                              const T* der, G* grad, uint32_t lane) {
   const uint32_t nout = 1u << op.rc, ny = 1u << op.ry;
   const BitMap p1(op.p1), p2(op.p2), y1(op.y1), y2(op.y2);

@@ -121,8 +121,9 @@ __device__ __forceinline__ T* locate(uint32_t off, bool global, T* gbase, T* tab
 }
 
 template <typename T, int kTeams>
-__device__ __noinline__ void run_smem_task(const GraphProgDev& prog, const GTask& task, T* table,
+__device__ __forceinline__ void run_smem_task(const GraphProgDev& prog, uint32_t t, T* table,
                               unsigned char* work, double* s_grad, const GTeam<kTeams>& team) {
+  const GTask& task = prog.tasks[t];
   const int P = prog.n_params;
   const int stride = 2 + 2 * P;
   for (int i = team.tid; i < 2 * P; i += team.size) s_grad[i] = 0.0;
@@ -172,8 +173,10 @@ __device__ __forceinline__ T ysum(const T* A, const T* B, uint32_t oa, uint32_t 
               cadd(cadd(acc[4], acc[5]), cadd(acc[6], acc[7])));
 }
 
-// Rows r0..r1 of a chunk whose summed index has NY values: R rows at a
-// time with every term's operands loaded before any product, so R * NY load
+// (The chunk code is inline throughout: a call saves up to 24 registers of 256
+// threads to local memory, 24 KB per task; run_chunk out of line made 7-regular
+// n=26 8 % slower, rows_fixed alone 1 %.)  Rows r0..r1 of a chunk whose
+// summed index has NY values: R rows at a time with every term's operands loaded before any product, so R * NY load
 // pairs are in flight per thread.  Rows past r1 load row r1 - 1 again and
 // store nothing.
 template <typename T, uint32_t R, uint32_t NY>
@@ -209,11 +212,50 @@ __device__ __forceinline__ void rows_unrolled(const T* A, const T* B, T* C, cons
   }
 }
 
+// Rows r0..r1 of a chunk with n_y >= 8 summed values, four rows at a time and two
+// summed values per pass: sixteen independent loads in flight per thread.
+template <typename T>
+__device__ __forceinline__ void rows_generic(const T* A, const T* B, T* C, const uint32_t* rowa,
+                                          const uint32_t* rowb, uint32_t a_lo, uint32_t b_lo,
+                                          const uint32_t* ya, const uint32_t* yb, uint32_t r0,
+                                          uint32_t r1, uint32_t rowlen, uint32_t n_y,
+                                          uint32_t tid) {
+  constexpr uint32_t R = 4;
+  for (uint32_t row = r0; row < r1; row += R) {
+    uint32_t oa[R], ob[R];
+    T acc[R];
+#pragma unroll
+    for (uint32_t r = 0; r < R; ++r) {
+      const uint32_t rr = min(row + r, r1 - 1) - r0;
+      oa[r] = rowa[rr] | a_lo;
+      ob[r] = rowb[rr] | b_lo;
+      acc[r] = czero<T>();
+    }
+    for (uint32_t y = 0; y < n_y; y += 2) {
+      const uint32_t ay0 = ya[y], by0 = yb[y], ay1 = ya[y + 1], by1 = yb[y + 1];
+      T av[R][2], bv[R][2];
+#pragma unroll
+      for (uint32_t r = 0; r < R; ++r) {
+        av[r][0] = A[oa[r] | ay0];
+        bv[r][0] = B[ob[r] | by0];
+        av[r][1] = A[oa[r] | ay1];
+        bv[r][1] = B[ob[r] | by1];
+      }
+#pragma unroll
+      for (uint32_t r = 0; r < R; ++r)
+        acc[r] = cfma(av[r][1], bv[r][1], cfma(av[r][0], bv[r][0], acc[r]));
+    }
+#pragma unroll
+    for (uint32_t r = 0; r < R; ++r)
+      if (row + r < r1) C[(row + r) * rowlen + tid] = acc[r];
+  }
+}
+
 // Rows of a GSF_ROWS step, four at a time: row k of a group reads A element
 // ia(k) and B element ib(k) of the group's distinct ones (GRS_ZX: A varies
 // with row bit 1, B with bit 0; GRS_ZZ: one A, four B; GRS_XX: four A, one
-// B), two summed values per pass, so a pass issues 8 (ZX) or 10 loads for 8
-// terms instead of 16.  nr is a multiple of four; rowc holds each row's
+// B), two summed values per pass (four for ZX in single precision), so a pass
+// issues 16 (ZX) or 10 loads for 16 or 8 terms.  nr is a multiple of four; rowc holds each row's
 // output offset.
 template <typename T, int kShare>
 __device__ __forceinline__ void rows_shared(const T* A, const T* B, T* C, const uint32_t* rowa,
@@ -223,6 +265,7 @@ __device__ __forceinline__ void rows_shared(const T* A, const T* B, T* C, const 
                                             uint32_t tid) {
   constexpr int NA = kShare == GRS_ZZ ? 1 : (kShare == GRS_ZX ? 2 : 4);
   constexpr int NB = kShare == GRS_XX ? 1 : (kShare == GRS_ZX ? 2 : 4);
+  constexpr int Y = kShare == GRS_ZX && sizeof(T) == 8 ? 4 : 2;
   auto ia = [](int k) { return kShare == GRS_ZZ ? 0 : (kShare == GRS_ZX ? k >> 1 : k); };
   auto ib = [](int k) { return kShare == GRS_XX ? 0 : (kShare == GRS_ZX ? k & 1 : k); };
   for (uint32_t r = 0; r < nr; r += 4) {
@@ -234,22 +277,20 @@ __device__ __forceinline__ void rows_shared(const T* A, const T* B, T* C, const 
     T acc[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) acc[k] = czero<T>();
-    for (uint32_t y = 0; y < n_y; y += 2) {
-      const uint32_t ay0 = ya[y], by0 = yb[y], ay1 = ya[y + 1], by1 = yb[y + 1];
-      T av[NA][2], bv[NB][2];
+    for (uint32_t y = 0; y < n_y; y += Y) {
+      T av[NA][Y], bv[NB][Y];
 #pragma unroll
-      for (int i = 0; i < NA; ++i) {
-        av[i][0] = A[oa[i] | ay0];
-        av[i][1] = A[oa[i] | ay1];
+      for (int u = 0; u < Y; ++u) {
+        const uint32_t ay = ya[y + u], by = yb[y + u];
+#pragma unroll
+        for (int i = 0; i < NA; ++i) av[i][u] = A[oa[i] | ay];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) bv[i][u] = B[ob[i] | by];
       }
 #pragma unroll
-      for (int i = 0; i < NB; ++i) {
-        bv[i][0] = B[ob[i] | by0];
-        bv[i][1] = B[ob[i] | by1];
-      }
+      for (int u = 0; u < Y; ++u)
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        acc[k] = cfma(av[ia(k)][1], bv[ib(k)][1], cfma(av[ia(k)][0], bv[ib(k)][0], acc[k]));
+        for (int k = 0; k < 4; ++k) acc[k] = cfma(av[ia(k)][u], bv[ib(k)][u], acc[k]);
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) C[rowc[r + k] + tid] = acc[k];
@@ -258,10 +299,9 @@ __device__ __forceinline__ void rows_shared(const T* A, const T* B, T* C, const 
 
 // Rows of a GRS_FIXA / GRS_FIXB step (1, 2 or 4 summed values): groups of 2^G
 // rows read the fixed operand S once per summed value and the other operand
-// O per row, 2^G x NY loads of O in flight per thread.  Kept out of line so
-// its registers do not weigh on the rest of the chunk code.
+// O per row, 2^G x NY loads of O in flight per thread.
 template <typename T, uint32_t NY, uint32_t G>
-__device__ __noinline__ void rows_fixed(const T* S, const T* O, T* C, const uint32_t* rows_s,
+__device__ __forceinline__ void rows_fixed(const T* S, const T* O, T* C, const uint32_t* rows_s,
                                         const uint32_t* rows_o, const uint32_t* rowc,
                                         uint32_t s_lo, uint32_t o_lo, const uint32_t* ys,
                                         const uint32_t* yo, uint32_t nr, uint32_t tid) {
@@ -712,10 +752,9 @@ __device__ __forceinline__ void rows_pair(const float2* A, const float2* B, floa
 
 // rows_shared for complex64 steps with paired loads (summed bit 0 is bit 0
 // of both operands): two 16-byte pairs per distinct element and pass, so a
-// ZX group of four rows issues 8 loads for 16 terms.  Out of line, like
-// rows_fixed.
+// ZX group of four rows issues 8 loads for 16 terms.
 template <int kShare>
-__device__ __noinline__ void rows_shared_pair(const float2* A, const float2* B, float2* C,
+__device__ __forceinline__ void rows_shared_pair(const float2* A, const float2* B, float2* C,
                                               const uint32_t* rowa, const uint32_t* rowb,
                                               const uint32_t* rowc, uint32_t a_lo, uint32_t b_lo,
                                               const uint32_t* ya, const uint32_t* yb,
@@ -809,6 +848,144 @@ __device__ __forceinline__ T warp_ysum(const T* A, const T* B, uint32_t oa, uint
   return sum;
 }
 
+// ---- staged rows: long sums in few tasks ------------------------------------
+
+// One element from global to shared memory, asynchronously.
+__device__ __forceinline__ void cp_async_elem(float2* dst, const float2* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_elem(double2* dst, const double2* src) {
+  cp_async16(dst, src);
+}
+
+// The terms of one batch added to a thread's accumulators: J of them, each of G
+// consecutive values in every eight (a lone one of J = 1 starts at value l).
+template <typename T, int J, int G>
+__device__ __forceinline__ void add_batch(const T* a, const T* b, uint32_t ea, uint32_t eb,
+                                          uint32_t n, uint32_t l, T* acc) {
+#pragma unroll 4
+  for (uint32_t y = 0; y < n; y += 8) {
+#pragma unroll
+    for (int k = 0; k < J; ++k) {
+      const uint32_t v = y + (J > 1 ? (uint32_t)k * G : l);
+#pragma unroll
+      for (int g = 0; g < G; ++g) acc[k] = cfma(a[(v + g) * ea], b[(v + g) * eb], acc[k]);
+    }
+  }
+}
+
+// Outputs [row 2^share, (row + 1) 2^share) of a GSF_STAGE step.  Their distinct
+// operand elements for 2^stage_y summed values are copied into one half of the
+// stage while the other half is added up, so a batch's loads are all in flight
+// at once; the sum itself is a chain of two dependent multiply-adds per term and
+// component.  Terms are added as the step's row form adds them: sequentially, in
+// eight accumulators (folded every kYTab values) or in four of pairs.  With few
+// outputs the accumulators go to lanes of their own.  Bound by the copies' round
+// trips (about 1.5 us a batch): 0.1 to 0.2 T multiply-adds/s over the device
+// against the row forms' 0.9, but a step of 2048 outputs x 2048 terms (two row
+// tasks) takes tens of us instead of 509: dense p=2 n=100 in split BF16 717 ->
+// 391 us, value + gradient 1106 -> 963 us.
+template <typename T, int kTeams>
+__device__ __forceinline__ void run_stage_row(const GStep& st, const T* A, const T* B, T* C,
+                                           uint32_t row, unsigned char* work,
+                                           const GTeam<kTeams>& team) {
+  const uint32_t tid = team.tid;
+  const uint32_t rowlen = 1u << st.share;
+  const uint32_t ny = 1u << st.ry, ly = st.stage_y, Y = 1u << ly;
+  uint32_t* offa = reinterpret_cast<uint32_t*>(work);
+  uint32_t* offb = offa + 256;
+  uint2* ytab = reinterpret_cast<uint2*>(work + kStageOffsets);   // two batches
+  T* buf = reinterpret_cast<T*>(work + kStageHead);
+  // low output bits held by each operand; this thread's place in the footprints
+  uint32_t ma = 0, mb = 0;
+  for (uint32_t i = 0; (1u << i) < rowlen; ++i) {
+    if (runs_offset(st.ca, 1u << i)) ma |= 1u << i;
+    if (runs_offset(st.cb, 1u << i)) mb |= 1u << i;
+  }
+  const uint32_t la = __popc(ma), lb = __popc(mb), ea = 1u << la, eb = 1u << lb;
+  const uint32_t n_acc = st.flags & GSF_SUM8 ? 8u : st.flags & GSF_SUM_PAIR4 ? 4u : 1u;
+  const bool lanes = n_acc > 1 && rowlen * n_acc <= kGraphBlock;   // an accumulator per thread
+  const uint32_t c = tid & (rowlen - 1), l = tid / rowlen;
+  const bool active = lanes ? l < n_acc : l == 0;
+  uint32_t fa = 0, fb = 0, pa = 0, pb = 0;   // gather of c, scatter of tid
+  for (uint32_t i = 0, ka = 0, kb = 0; i < 8; ++i) {
+    if ((ma >> i) & 1u) {
+      fa |= ((c >> i) & 1u) << ka;
+      pa |= ((tid >> ka++) & 1u) << i;
+    }
+    if ((mb >> i) & 1u) {
+      fb |= ((c >> i) & 1u) << kb;
+      pb |= ((tid >> kb++) & 1u) << i;
+    }
+  }
+  if (tid < ea) offa[tid] = runs_offset(st.ca, row * rowlen | pa);
+  if (tid < eb) offb[tid] = runs_offset(st.cb, row * rowlen | pb);
+  for (uint32_t y = tid; y < 2 * Y && y < ny; y += kGraphBlock)
+    ytab[y] = make_uint2(runs_offset(st.ya, y), runs_offset(st.yb, y));
+  team.sync();
+  const uint32_t half = Y * (ea + eb);
+  auto issue = [&](uint32_t k) {
+    T* dst = buf + (k & 1u) * half;
+    const uint2* yt = ytab + (k & 1u) * Y;
+    for (uint32_t i = tid; i < Y * ea; i += kGraphBlock)
+      cp_async_elem(dst + i, A + (offa[i & (ea - 1)] | yt[i >> la].x));
+    dst += Y * ea;
+    for (uint32_t i = tid; i < Y * eb; i += kGraphBlock)
+      cp_async_elem(dst + i, B + (offb[i & (eb - 1)] | yt[i >> lb].y));
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  T acc[8], total = czero<T>();
+#pragma unroll
+  for (int u = 0; u < 8; ++u) acc[u] = czero<T>();
+  const uint32_t nb = ny >> ly, fold = ny <= kYTab ? nb : kYTab >> ly;
+  issue(0);
+  for (uint32_t k = 0; k < nb; ++k) {
+    if (k + 1 < nb) {
+      issue(k + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    // offsets of the batch after next, in the slots of this one's (already used)
+    if (k + 2 < nb)
+      for (uint32_t y = tid; y < Y; y += kGraphBlock) {
+        const uint32_t yy = (k + 2) * Y + y;
+        ytab[(k & 1u) * Y + y] = make_uint2(runs_offset(st.ya, yy), runs_offset(st.yb, yy));
+      }
+    team.sync();
+    if (active) {
+      const T* a = buf + (k & 1u) * half + fa;
+      const T* b = buf + (k & 1u) * half + Y * ea + fb;
+      if (n_acc == 1) add_batch<T, 1, 8>(a, b, ea, eb, Y, 0, acc);
+      else if (n_acc == 4)
+        lanes ? add_batch<T, 1, 2>(a, b, ea, eb, Y, 2 * l, acc)
+              : add_batch<T, 4, 2>(a, b, ea, eb, Y, 0, acc);
+      else
+        lanes ? add_batch<T, 1, 1>(a, b, ea, eb, Y, l, acc)
+              : add_batch<T, 8, 1>(a, b, ea, eb, Y, 0, acc);
+    }
+    team.sync();
+    if ((k + 1) % fold == 0) {
+      if (lanes) {
+        // accumulator l of output c, through the batch just used
+        T* red = buf + (k & 1u) * half;
+        if (active) red[l * rowlen + c] = acc[0];
+        team.sync();
+        if (l == 0)
+          for (uint32_t u = 1; u < n_acc; ++u) acc[u] = red[u * rowlen + c];
+        team.sync();
+      }
+      T sum = acc[0];
+      if (n_acc > 1) sum = cadd(cadd(acc[0], acc[1]), cadd(acc[2], acc[3]));
+      if (n_acc == 8) sum = cadd(sum, cadd(cadd(acc[4], acc[5]), cadd(acc[6], acc[7])));
+      total = cadd(total, sum);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc[u] = czero<T>();
+    }
+  }
+  if (l == 0) C[row * rowlen + c] = total;
+}
+
 template <typename T, int kTeams, bool kTile>
 __device__ void run_chunk(const GraphProgDev& prog, const GTask& task, T* table,
                           unsigned char* work, GStep& s_step, int& s_last,
@@ -836,6 +1013,11 @@ __device__ void run_chunk(const GraphProgDev& prog, const GTask& task, T* table,
   const uint32_t nout = 1u << st.rc;
   const uint64_t ny = 1ull << st.ry;
 
+  if (st.flags & GSF_STAGE) {
+    run_stage_row<T, kTeams>(st, A, B, gb + st.c_off, task.b, work, team);
+    signal_done(prog, st.done_ctr, team);
+    return;
+  }
   if (!(st.flags & GSF_SPLIT)) {
     T* C = gb + st.c_off;
     const uint32_t rowlen = nout < kGRow ? nout : kGRow;
@@ -861,7 +1043,6 @@ __device__ void run_chunk(const GraphProgDev& prog, const GTask& task, T* table,
         rowc[r] = o * rowlen;
       }
       team.sync();
-      constexpr uint32_t R = 4;
       const uint32_t n_y = (uint32_t)ny;
       if (active && shared_rows && st.share >= GRS_FIXA) {
         rows_fixed_dispatch(A, B, C, rowa, rowb, rowc, a_lo, b_lo, ya, yb, r1 - r0, n_y,
@@ -886,8 +1067,8 @@ __device__ void run_chunk(const GraphProgDev& prog, const GTask& task, T* table,
       } else if (active && (st.flags & GSF_YPAIR) &&
           rows_paired(A, B, C, rowa, rowb, a_lo, b_lo, ya, yb, r0, r1, rowlen, tid, n_y)) {
         // complex64 element pairs along summed bit 0
-      } else if (active && r1 - r0 < R) {
-        // few rows with long sums: the summed index unrolled instead
+      } else if (active && (st.flags & GSF_SUM8)) {
+        // rows with long sums: the summed index unrolled instead
         for (uint32_t row = r0; row < r1; ++row)
           C[row * rowlen + tid] = ysum(A, B, rowa[row - r0] | a_lo, rowb[row - r0] | b_lo, ya,
                                        yb, 0u, n_y, 1u);
@@ -898,36 +1079,7 @@ __device__ void run_chunk(const GraphProgDev& prog, const GTask& task, T* table,
       } else if (active && n_y == 4) {
         rows_unrolled<T, 2, 4>(A, B, C, rowa, rowb, a_lo, b_lo, ya, yb, r0, r1, rowlen, tid);
       } else if (active) {
-        // four rows at a time: eight independent loads in flight per thread
-        for (uint32_t row = r0; row < r1; row += R) {
-          uint32_t oa[R], ob[R];
-          T acc[R];
-#pragma unroll
-          for (uint32_t r = 0; r < R; ++r) {
-            const uint32_t rr = min(row + r, r1 - 1) - r0;
-            oa[r] = rowa[rr] | a_lo;
-            ob[r] = rowb[rr] | b_lo;
-            acc[r] = czero<T>();
-          }
-          // two summed values per pass (n_y >= 8 here): sixteen loads in flight
-          for (uint32_t y = 0; y < n_y; y += 2) {
-            const uint32_t ay0 = ya[y], by0 = yb[y], ay1 = ya[y + 1], by1 = yb[y + 1];
-            T av[R][2], bv[R][2];
-#pragma unroll
-            for (uint32_t r = 0; r < R; ++r) {
-              av[r][0] = A[oa[r] | ay0];
-              bv[r][0] = B[ob[r] | by0];
-              av[r][1] = A[oa[r] | ay1];
-              bv[r][1] = B[ob[r] | by1];
-            }
-#pragma unroll
-            for (uint32_t r = 0; r < R; ++r)
-              acc[r] = cfma(av[r][1], bv[r][1], cfma(av[r][0], bv[r][0], acc[r]));
-          }
-#pragma unroll
-          for (uint32_t r = 0; r < R; ++r)
-            if (row + r < r1) C[(row + r) * rowlen + tid] = acc[r];
-        }
+        rows_generic(A, B, C, rowa, rowb, a_lo, b_lo, ya, yb, r0, r1, rowlen, n_y, tid);
       }
     } else {
       // one row per chunk; the summed index in passes of kYTab values
@@ -1316,7 +1468,7 @@ __global__ void __launch_bounds__(kGraphBlock*(kTc ? 4 : 1),
     if (!s_flag[team.id]) break;
     const GTask task = prog.tasks[s_task[team.id]];
     if (task.kind == GT_SMEM) {
-      run_smem_task<T, kTeams>(prog, task, table, work, s_grad[team.id], team);
+      run_smem_task<T, kTeams>(prog, s_task[team.id], table, work, s_grad[team.id], team);
     } else if (task.kind == GT_CHUNK) {
       run_chunk<T, kTeams, kTile>(prog, task, table, work, s_step[team.id], s_last[team.id], team);
     } else if (kTc && prog.tmem_cols > 0) {

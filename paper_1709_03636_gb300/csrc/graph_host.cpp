@@ -26,7 +26,7 @@ uint64_t runs_max(const GRuns& r, uint32_t bits);
 // its class of step (by summed bits; split reductions apart) divided over
 // the resident teams, plus a fixed cost per task.
 double task_time_estimate(const GUnit& u, size_t elem, int teams) {
-  if (u.kind == GT_SMEM) return 30000.0;
+  if (u.kind == GT_SMEM) return 6000.0 + 0.5 * u.smem_cycles;   // (2 cycles a ns)
   if (u.kind == GT_TC) return 5000.0;
   const GStep& st = u.step;
   const double a = (st.flags & GSF_A_TABLE)
@@ -46,8 +46,14 @@ double task_time_estimate(const GUnit& u, size_t elem, int teams) {
   else if ((st.flags & GSF_ROWS) && (st.share == GRS_FIXA || st.share == GRS_FIXB) && ry <= 2)
     rate = kRateFixed[ry];
   else if ((st.flags & GSF_ROWS) && ry >= 3) rate = kRateShared[ry];
+  if (st.flags & GSF_STAGE) return 3000.0 + std::ldexp(12.0, st.ry);   // about 12 ns a term
   const double bytes = (double)elem * (a + b + c) / std::max<uint32_t>(st.n_chunks, 1);
-  return 1000.0 + bytes * teams / rate;
+  // A row task of few others is bound by its loads' latency.  (This and the
+  // subtree estimate put long tasks early: dense p=2 n=100 value + gradient 1.50
+  // -> 1.25 ms.)
+  const double latency =
+      st.flags & GSF_SPLIT ? 0.0 : 1000.0 + std::ldexp(70.0 * st.chunk, st.ry);
+  return std::max(1000.0 + bytes * teams / rate, latency);
 }
 
 WaveHost assemble_wave(const std::vector<int>& nets, const std::vector<NetGraph>& graphs,
@@ -325,6 +331,21 @@ void validate_wave(const WaveHost& w, uint32_t table_elems, uint32_t arena_elems
       if ((st.flags & GSF_LANES_Y) && !(st.flags & GSF_SPLIT))
         fail(QTC_ERR_INVALID, "internal: lanes over the summed index outside a split step");
     }
+    if (st.flags & GSF_STAGE) {
+      uint32_t fa = 1, fb = 1;
+      for (uint32_t i = 0; i < st.share; ++i) {
+        if (runs_offset_host(st.ca, 1ull << i)) fa *= 2;
+        if (runs_offset_host(st.cb, 1ull << i)) fb *= 2;
+      }
+      if ((st.flags & (GSF_SPLIT | GSF_TILE | GSF_ROWS | GSF_YPAIR | GSF_LANES_Y | GSF_A_TABLE |
+                       GSF_B_TABLE)) ||
+          st.share > 8 || st.share > st.rc || st.chunk != 1 ||
+          st.n_chunks != (1u << (st.rc - st.share)) || st.stage_y < 4 || st.stage_y > st.ry ||
+          (1u << st.stage_y) > kStageMaxY ||
+          kStageHead + (2ull << st.stage_y) * (fa + fb) * elem_of_wave > kStageBytes ||
+          kStageBytes > work_bytes)
+        fail(QTC_ERR_INVALID, "internal: staged rows on an unfit step");
+    }
     if (st.flags & GSF_ROWS) {
       // rows in groups along output bits that one operand lacks; the row
       // order a bijection of the row bits
@@ -468,6 +489,12 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
     return best;
   };
   const TreeModel model = tree_model(hp.dtype);
+  // A network's steps are cut finer when few networks share the device: one p=3
+  // edge network 551 -> 456 us.  With 120 networks the finer tasks cost more than
+  // the shorter chains give (p=3 n=60 4.50 -> 4.85 ms).
+  const uint32_t teams = (uint32_t)opts.sm_count * 4;
+  lim.min_chunks = std::min(std::max(teams / (uint32_t)N, 1u), teams);
+  if (lim.min_chunks < 32) lim.min_chunks = 1;
   std::vector<NetGraph> graphs(N);
   std::vector<Error> errors(N, Error{QTC_OK, ""});
   auto lower_one = [&](int i) {
@@ -478,7 +505,7 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
       GUnit u;
       u.kind = GT_SMEM;
       u.ops = std::move(ln.ops);
-      schedule_cta_ops(u.ops, hp.table_elems, kGraphWarps);
+      u.smem_cycles = schedule_cta_ops(u.ops, hp.table_elems, kGraphWarps);
       u.arena_elems = ln.arena_elems;
       graphs[i].units.push_back(std::move(u));
       return;

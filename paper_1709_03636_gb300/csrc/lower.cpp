@@ -274,10 +274,15 @@ uint32_t log2_floor(uint64_t x) {
 
 // Fills the bit maps and chunking of C = sum over (A u B) - C of A * B.
 // force_split: always reduce over chunks of the summed index (leaf adjoints).
-// A chunk task covers about 2^task_terms_log2 multiply-adds.
+// A chunk task covers about 2^task_terms_log2 multiply-adds, fewer where the
+// step would have less than `min_chunks` of them; may_stage: the staged form may
+// be taken.  How a row's terms are added
+// (sequentially, in eight accumulators, in four of pairs) depends on the step
+// alone, not on how it is cut.
 bool encode_gstep(GStep& g, const std::vector<int>& lc, const std::vector<int>& la,
                   const std::vector<int>& lb, bool force_split, int task_terms_log2,
-                  bool a_global, bool b_global, std::string* why) {
+                  uint32_t min_chunks, bool may_stage, size_t elem, bool a_global,
+                  bool b_global, std::string* why) {
   std::vector<int> pa, pb, ya, yb;
   for (int x : lc) {
     pa.push_back(pos_in(la, x));
@@ -398,6 +403,56 @@ bool encode_gstep(GStep& g, const std::vector<int>& lc, const std::vector<int>& 
         g.n_chunks = (uint32_t)(nrows / per);
         g.flags |= GSF_ROWS;
       }
+    }
+  }
+  if (g.flags & GSF_SPLIT) return true;
+  const uint64_t rowlen = std::min<uint64_t>(nout, kGRow), nrows = nout / rowlen;
+  const bool pairs = (g.flags & GSF_YPAIR) && elem == 8 && ny <= kYTab;
+  if (ny > kYTab || (!(g.flags & GSF_ROWS) && !pairs && ny >= 8 && g.chunk < 4))
+    g.flags |= GSF_SUM8;
+  // Long sums in few tasks: 32 to 256 outputs per task, operands staged in
+  // batches (the row forms keep eight or sixteen loads in flight per thread, one
+  // memory round trip per two to eight terms: 60 to 140 ns per term and row of a
+  // task).  Staged tasks end sooner but take more of the teams' time in all (no
+  // operand is reused from registers), so only where a task would take long and
+  // the step has few: 2048 outputs x 2048 terms 509 us in two tasks before.
+  const double row_us = 1e-3 * (double)g.chunk * (double)ny *
+                        (pairs && !(g.flags & GSF_ROWS) ? 140 : g.flags & GSF_SUM8 ? 106 : 62);
+  const bool alone = min_chunks > 1;
+  if (a_global && b_global && ny >= 64 && may_stage &&
+      (alone ? row_us > 24 && g.n_chunks < min_chunks : row_us > 96 && g.n_chunks <= 32)) {
+    const uint32_t tasks = alone ? 256 : 32;
+    int lr = (int)log2_floor(rowlen), ly = 0;
+    auto batch = [&](int r) {
+      int ma = 0, mb = 0;
+      for (int i = 0; i < r; ++i) {
+        ma += pa[i] >= 0;
+        mb += pb[i] >= 0;
+      }
+      return stage_log2_y((1u << ma) + (1u << mb), (uint32_t)elem, g.ry);
+    };
+    while (lr > 5 && ((nout >> lr) < tasks || batch(lr) < 5)) --lr;
+    ly = batch(lr);
+    if (ly) {
+      const bool four = pairs && !(g.flags & GSF_ROWS);
+      g.flags &= (uint16_t)~(GSF_ROWS | GSF_YPAIR);
+      g.flags |= GSF_STAGE | (four ? GSF_SUM_PAIR4 : 0);
+      g.share = (uint8_t)lr;
+      g.stage_y = (uint8_t)ly;
+      g.chunk = 1;
+      g.n_chunks = (uint32_t)(nout >> lr);
+      return true;
+    }
+  }
+  // other steps of few tasks: fewer rows per task, whole groups of shared rows
+  const uint64_t group = !(g.flags & GSF_ROWS) ? (ny == 1 ? 8 : 4)
+                         : g.share >= GRS_FIXA ? 1ull << grs_fix_bits((uint32_t)ny) : 4;
+  if (g.n_chunks < min_chunks && g.chunk > group) {
+    const uint64_t per =
+        std::max<uint64_t>(group, 1ull << log2_floor(std::max<uint64_t>(1, nrows / min_chunks)));
+    if (per < g.chunk) {
+      g.chunk = (uint32_t)per;
+      g.n_chunks = (uint32_t)((nrows + per - 1) / per);
     }
   }
   return true;
@@ -813,12 +868,13 @@ NetGraph lower_graph(const Plan& plan, const std::vector<int>& leaf_gate,
     }
     u.arena_elems = place_arena(ops, buf_size, table_elems, u.ops);
     if (u.arena_elems > lim.arena_elems) return false;
-    schedule_cta_ops(u.ops, table_elems, kGraphWarps);
+    u.smem_cycles = schedule_cta_ops(u.ops, table_elems, kGraphWarps);
     const int id = add_unit(std::move(u));
     if (!reverse && in_global[L + rs]) producer_val[L + rs] = id;
     return true;
   };
 
+  bool in_adjoint = false;
   auto gstep_unit = [&](int lc_t, const std::vector<int>& lc, int a, const std::vector<int>& la,
                         Ref ra, int b, const std::vector<int>& lb, Ref rb, int64_t c_off,
                         std::vector<int> deps, int leaf_for_grad) -> int {
@@ -836,8 +892,9 @@ NetGraph lower_graph(const Plan& plan, const std::vector<int>& leaf_gate,
     u.kind = GT_CHUNK;
     std::memset(&u.step, 0, sizeof u.step);
     std::string why;
-    if (!encode_gstep(u.step, lc, la, lb, leaf_for_grad >= 0, lim.task_terms_log2, ra.global,
-                      rb.global, &why)) {
+    if (!encode_gstep(u.step, lc, la, lb, leaf_for_grad >= 0, lim.task_terms_log2,
+                      lim.tile_mode ? 1u : lim.min_chunks,
+                      lim.tile_mode == 0 && (!in_adjoint || lim.min_chunks > 1), lim.elem, ra.global, rb.global, &why)) {
       ng.fits = false;
       ng.why = why;
       return -1;
@@ -851,7 +908,7 @@ NetGraph lower_graph(const Plan& plan, const std::vector<int>& leaf_gate,
     if (tm == 2 || tm == 4 || (tm == 1 && (two_global || (u.step.flags & GSF_SPLIT))) ||
         (tm == 3 && u.step.ry >= 3)) {
       GStep tiled = u.step;
-      tiled.flags &= (uint16_t)~(GSF_SPLIT | GSF_YPAIR | GSF_LANES_Y);
+      tiled.flags &= (uint16_t)~(GSF_SPLIT | GSF_YPAIR | GSF_LANES_Y | GSF_SUM8);
       if (encode_tile(tiled, lc, la, lb, !ra.global, !rb.global, lim.elem, lim.task_terms_log2,
                       tm >= 3))
         u.step = tiled;
@@ -999,6 +1056,7 @@ NetGraph lower_graph(const Plan& plan, const std::vector<int>& leaf_gate,
   };
 
   // ---- adjoint sweep, in reverse step order ----
+  in_adjoint = true;
   if (want_grad && need_grad[root]) {
     int entered = n_seg - 1;
     for (int s = S - 1; s >= 0; --s) {

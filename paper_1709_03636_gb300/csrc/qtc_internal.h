@@ -184,7 +184,8 @@ void build_warp_steps(const std::vector<SOp>& ops, uint32_t table_elems, uint32_
 void validate_warp_steps(const WStep* steps, size_t n, uint32_t team_elems, int n_params);
 
 // Puts a task's ops into levels for a team of n_warps warps (cta_program.cpp).
-void schedule_cta_ops(std::vector<SOp>& ops, uint32_t table_elems, int n_warps);
+// Returns the cycles that its levels are expected to take.
+double schedule_cta_ops(std::vector<SOp>& ops, uint32_t table_elems, int n_warps);
 // Host check of such a program: every access against its buffer, no conflict
 // within a level, one warp per gradient slot.
 void validate_cta_ops(const SOp* ops, size_t n, uint32_t table_elems, uint32_t arena_elems,
@@ -230,6 +231,7 @@ struct GraphLimits {
                                      // memory, 2 every step that tiles; read in place:
                                      // 3 steps summing >= 3 labels, 4 every step that tiles
   size_t elem = 8;                   // bytes per element
+  uint32_t min_chunks = 1;           // tasks a global step is cut into where its rows allow
 };
 
 // Tile form of a global step (tile_plan.cpp): fills g.tile, g.n_chunks and
@@ -244,6 +246,7 @@ size_t tile_region_bytes(const GStep& g, size_t elem);
 // plain contraction over its bit maps: the largest absolute difference.
 double emulate_tile_step(const GStep& g, uint64_t seed);
 double emulate_rows_step(const GStep& g, uint64_t seed);
+double emulate_stage_step(const GStep& g, uint64_t seed);
 
 // A unit is one shared-memory subtree task or one global step (its chunks);
 // its counter reaches `target` when it is complete.
@@ -253,6 +256,7 @@ struct GUnit {
   GStep step{};                      // GT_CHUNK
   TStep tstep{};                     // GT_TC
   uint32_t arena_elems = 0;
+  double smem_cycles = 0;            // GT_SMEM: expected
   std::vector<int> deps;             // units that must be complete first
   int depth = 0;
   uint32_t target = 1;

@@ -427,4 +427,66 @@ double emulate_rows_step(const GStep& g, uint64_t seed) {
   return err;
 }
 
+// The staged form of a row (footprints of both operands by batches of summed
+// values) against the plain contraction.
+double emulate_stage_step(const GStep& g, uint64_t seed) {
+  const uint64_t ra = (apply(g.ca, (1ull << g.rc) - 1) | apply(g.ya, (1ull << g.ry) - 1)) + 1;
+  const uint64_t rb = (apply(g.cb, (1ull << g.rc) - 1) | apply(g.yb, (1ull << g.ry) - 1)) + 1;
+  SplitMix64 rng(seed);
+  auto draw = [&]() { return std::complex<double>((double)(rng.next() >> 11) * 0x1p-53 - 0.5,
+                                                  (double)(rng.next() >> 11) * 0x1p-53 - 0.5); };
+  std::vector<std::complex<double>> A(ra), B(rb);
+  for (auto& x : A) x = draw();
+  for (auto& x : B) x = draw();
+  const uint64_t rowlen = 1ull << g.share, ny = 1ull << g.ry;
+  auto mask_of = [&](const GRuns& r) {
+    uint32_t m = 0;
+    for (uint32_t i = 0; (1ull << i) < rowlen; ++i)
+      if (apply(r, 1ull << i)) m |= 1u << i;
+    return m;
+  };
+  auto scatter = [](uint32_t j, uint32_t m) {   // bits of j to the set bits of m
+    uint32_t v = 0;
+    for (uint32_t i = 0; m >> i; ++i)
+      if ((m >> i) & 1u) {
+        v |= (j & 1u) << i;
+        j >>= 1;
+      }
+    return v;
+  };
+  auto gather = [](uint32_t c, uint32_t m) {
+    uint32_t v = 0, k = 0;
+    for (uint32_t i = 0; m >> i; ++i)
+      if ((m >> i) & 1u) v |= ((c >> i) & 1u) << k++;
+    return v;
+  };
+  const uint32_t ma = mask_of(g.ca), mb = mask_of(g.cb);
+  const uint32_t ea = 1u << __builtin_popcount(ma), eb = 1u << __builtin_popcount(mb);
+  const uint32_t Y = 1u << g.stage_y;
+  std::vector<std::complex<double>> sa((size_t)Y * ea), sb((size_t)Y * eb);
+  double err = 0;
+  for (uint64_t row = 0; row < g.n_chunks; ++row) {
+    std::vector<std::complex<double>> acc(rowlen, 0.0);
+    for (uint64_t y0 = 0; y0 < ny; y0 += Y) {
+      for (uint32_t y = 0; y < Y; ++y) {
+        for (uint32_t j = 0; j < ea; ++j)
+          sa[(size_t)y * ea + j] = A[apply(g.ca, row * rowlen | scatter(j, ma)) | apply(g.ya, y0 + y)];
+        for (uint32_t j = 0; j < eb; ++j)
+          sb[(size_t)y * eb + j] = B[apply(g.cb, row * rowlen | scatter(j, mb)) | apply(g.yb, y0 + y)];
+      }
+      for (uint32_t c = 0; c < rowlen; ++c)
+        for (uint32_t y = 0; y < Y; ++y)
+          acc[c] += sa[(size_t)y * ea + gather(c, ma)] * sb[(size_t)y * eb + gather(c, mb)];
+    }
+    for (uint32_t c = 0; c < rowlen; ++c) {
+      std::complex<double> ref = 0.0;
+      const uint64_t o = row * rowlen + c;
+      for (uint64_t y = 0; y < ny; ++y)
+        ref += A[apply(g.ca, o) | apply(g.ya, y)] * B[apply(g.cb, o) | apply(g.yb, y)];
+      err = std::max(err, std::abs(ref - acc[c]));
+    }
+  }
+  return err;
+}
+
 }  // namespace qtc
