@@ -427,14 +427,16 @@ def _autograd():
             out = torch.empty(2 + 2 * p + len(batch.edges), dtype=torch.float64,
                               device=prm.device)
             qaoa_expectation_device(engine, batch, prm, out, dtype, want_grad=True)
-            ctx.save_for_backward(out[1:1 + 2 * p].clone())
+            ctx.save_for_backward(out)
             ctx.param_device = params.device
-            return out[0].clone().to(device=params.device, dtype=params.dtype)
+            ctx.p = p
+            # one copy that nothing else holds, cast and moved at once
+            return out[0].to(device=params.device, dtype=params.dtype, copy=True)
 
         @staticmethod
         def backward(ctx, grad_out):
-            (grad,) = ctx.saved_tensors
-            g = grad.to(device=ctx.param_device, dtype=grad_out.dtype)
+            (out,) = ctx.saved_tensors
+            g = out[1:1 + 2 * ctx.p].to(device=ctx.param_device, dtype=grad_out.dtype)
             return grad_out * g, None, None, None
 
     return QAOAExpectation
