@@ -1568,15 +1568,9 @@ static SvPrepared& sv_prepare(qtc_engine* e, qtc_circuit* c, cudaStream_t s) {
   p.acc = (double*)e->alloc(sizeof(double) * (1 + cc.edges.size()));
   void* scratch = e->alloc((size_t)16 * (cc.p * (cc.edges.size() + 1) + cc.p + 2));
   for (int d = 0; d < 2; ++d) {
-    int lo[16], len[16], rl[16];
-    const int passes = sv_passes(cc.n, sv_tile_bits(d), lo, len, rl);
-    const int l = passes - 1;
     p.tabs[d].scratch = scratch;
-    p.tabs[d].wcut_first =
-        upload(e, sv_cut_table(adj, cc.n, lo[0], len[0], rl[0]), s, "upload cut table");
-    p.tabs[d].wcut_last =
-        passes > 1 ? upload(e, sv_cut_table(adj, cc.n, lo[l], len[l], rl[l]), s, "upload cut table")
-                   : p.tabs[d].wcut_first;
+    p.tabs[d].wcut = cc.n < sv_tile_bits(d)
+                         ? upload(e, sv_cut_table(adj), s, "upload cut table") : nullptr;
   }
   cuda_check(cudaStreamSynchronize(s), "prepare sync");
   c->sv.push_back(p);

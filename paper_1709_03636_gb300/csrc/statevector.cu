@@ -5,14 +5,13 @@
 // <Z_a Z_b> per edge.
 //
 // Layout: qubit q is bit q of the element index.  A pass moves tiles of 2^tb
-// elements through shared memory (64 KB: 2^13 complex64 or 2^12 complex128,
-// two or three CTAs per SM).  Pass 0 of a layer holds qubits 0..tb-1
-// (contiguous tiles) and applies the layer's phase on load; every further pass
-// mixes its own group of qubits and carries as many low qubits along
-// (unmixed) as fill the tile, so tiles stay full and rows contiguous.  The
-// qubits above pass 0 are split evenly over the fewest passes.  The mixer's
-// 2x2 rotation is applied to the pass's own qubits on elements held in
-// registers (and lane bits by shuffles).
+// elements (64 KB: 2^13 complex64 or 2^12 complex128, two CTAs per SM) through
+// registers.  Pass 0 of a layer holds qubits 0..tb-1 (contiguous tiles) and
+// applies the layer's phase on load; every further pass mixes its own group of
+// qubits and carries as many low qubits along (unmixed) as fill the tile, so
+// tiles stay full and rows contiguous.  The qubits above pass 0 are split evenly
+// over the fewest passes.  A state smaller than a tile is held in shared memory
+// by one CTA (sv_small_kernel).
 // The last pass of the last layer accumulates |psi|^2 cut(x).
 //
 // The rotation [[c, -i s], [-i s, c]] (c = cos beta, s = sin beta) is applied
@@ -24,12 +23,6 @@
 // <C>.  |f| >= 1/sqrt(2), so the stored amplitudes stay within
 // 2^(-n/2) .. 1 of the unit-norm state's scale.
 //
-// cut(x) without a loop over vertices: with the tile's vertices T and the
-// block's fixed bits f on the other vertices F,
-//   cut(x) = c0(f) + sum_{a in T} t_a coef_a(f) + W[t],
-// c0 = cut edges inside F plus edges from T to F whose F end is 1,
-// coef_a = deg_F(a) - 2 |N_F(a) and f|, W = cut edges inside T (a host-built
-// table per pass layout).  The linear term comes from two per-block tables.
 // The phase and rotation values are computed once per launch (FP64 angles).
 #include <cuda_runtime.h>
 
@@ -69,28 +62,15 @@ int sv_passes(int n, int tmax, int* lo, int* len, int* rl) {
   return 1 + k;
 }
 
-// Tile vertex of tile bit j for a pass (lo = 0: bits 0..len-1; else the
-// carried bits 0..rl-1 then lo..lo+len-1).
-static inline int tile_vertex(int lo, int rl, int j) {
-  return lo == 0 || j < rl ? j : lo + j - rl;
-}
-
-std::vector<uint16_t> sv_cut_table(const std::vector<uint32_t>& adj, int n, int lo, int len,
-                                   int rl) {
-  const int tb = lo == 0 ? len : rl + len;
-  std::vector<int> va(tb);
-  for (int j = 0; j < tb; ++j) va[j] = tile_vertex(lo, rl, j);
-  std::vector<std::pair<int, int>> inner;  // tile-internal edges as tile bit pairs
-  for (int j = 0; j < tb; ++j)
-    for (int k = j + 1; k < tb; ++k)
-      if ((adj[va[j]] >> va[k]) & 1u) inner.emplace_back(j, k);
-  std::vector<uint16_t> w((size_t)1 << tb);
-  for (uint32_t t = 0; t < (1u << tb); ++t) {
+std::vector<uint16_t> sv_cut_table(const std::vector<uint32_t>& adj) {
+  const int n = (int)adj.size();
+  std::vector<uint16_t> w((size_t)1 << n);
+  for (uint32_t t = 0; t < (1u << n); ++t) {
     int c = 0;
-    for (auto& e : inner) c += ((t >> e.first) ^ (t >> e.second)) & 1u;
+    for (int v = 0; v < n; ++v)
+      if ((t >> v) & 1u) c += __builtin_popcount(adj[v] & ~t);
     w[t] = (uint16_t)c;
   }
-  (void)n;
   return w;
 }
 
@@ -100,7 +80,7 @@ struct SvArgs {
   const uint32_t* adj;       // per qubit: bit mask of its neighbours (n <= 32)
   const void* phase;         // per layer m + 1 values exp(-i gamma (m - 2c) / 2)
   const void* rot;           // per layer (cos beta, sin beta)
-  const uint16_t* wcut;      // cut edges inside the tile (passes that need cut(x)), else null
+  const uint16_t* wcut;      // cut(x) of every x (states smaller than a tile), else null
   int layer;
   int lo, len, rl;           // pass: tile bits 0..len-1 (lo = 0) or 0..rl-1 and lo..lo+len-1
   int first;                 // 1: the state is |+>, do not read it
@@ -111,13 +91,6 @@ struct SvArgs {
   double* acc;               // [<C>, <ZZ> per edge]
 };
 
-// Per-block tables for cut(x) = c0(f) + sum_{a in T} t_a coef_a(f) + W[t]
-// (tile vertices T, the block's fixed bits f) and the layer's phase values.
-struct SvBlock {
-  int lo[128], hi[64], coef[16];
-  int c0;
-};
-
 template <typename T>
 __device__ __forceinline__ uint64_t sv_gidx(const SvArgs& a, uint64_t blk, uint32_t t) {
   if (a.lo == 0) return (blk << a.len) | t;
@@ -126,54 +99,6 @@ __device__ __forceinline__ uint64_t sv_gidx(const SvArgs& a, uint64_t blk, uint3
   const uint64_t below = blk & ((1ull << (a.lo - rl)) - 1);  // bits rl..lo-1
   const uint64_t above = blk >> (a.lo - rl);                   // bits lo+len..
   return low | (below << rl) | (mid << a.lo) | (above << (a.lo + a.len));
-}
-
-template <typename T>
-__device__ void sv_block_setup(const SvArgs& a, uint64_t blk, int tb, SvBlock& sb, T* s_phase) {
-  const int n = a.n;
-  const bool pass0 = a.lo == 0;
-  const int rl = a.rl;
-  if (a.wcut != nullptr) {
-    const uint32_t tsize = 1u << tb;
-    const uint32_t full = n == 32 ? 0xFFFFFFFFu : ((1u << n) - 1u);
-    const uint32_t tmask =
-        pass0 ? (uint32_t)(tsize - 1u) : (((1u << rl) - 1u) | (((1u << a.len) - 1u) << a.lo));
-    const uint32_t fm = full & ~tmask;
-    const uint32_t f = (uint32_t)sv_gidx<T>(a, blk, 0);  // fixed bits (tile bits zero)
-    if (threadIdx.x < 32) {
-      int part = 0;
-      const int v = threadIdx.x;
-      if (v < n) {
-        const uint32_t adj_f = a.adj[v] & fm;
-        if ((tmask >> v) & 1u)
-          part = __popc(adj_f & f);          // tile vertex at 0: edges to fixed ones at 1
-        else if ((f >> v) & 1u)
-          part = __popc(adj_f & ~f);         // fixed-fixed cut edges, counted from the 1 end
-      }
-      for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-      if (v == 0) sb.c0 = part;
-    }
-    if (threadIdx.x < (unsigned)tb) {
-      const int j = threadIdx.x;
-      const int v = pass0 || j < rl ? j : a.lo + j - rl;
-      const uint32_t adj_f = a.adj[v] & fm;
-      sb.coef[j] = __popc(adj_f) - 2 * __popc(adj_f & f);
-    }
-    __syncthreads();
-    if (threadIdx.x < 128) {
-      const int u = threadIdx.x;
-      int sl = 0, sh = 0;
-      for (int j = 0; j < 7 && j < tb; ++j) sl += ((u >> j) & 1) * sb.coef[j];
-      for (int j = 7; j < tb && u < 64; ++j) sh += ((u >> (j - 7)) & 1) * sb.coef[j];
-      sb.lo[u] = sl;
-      if (u < 64) sb.hi[u] = sh;
-    }
-  }
-  if (pass0) {
-    const T* ph = reinterpret_cast<const T*>(a.phase) + (size_t)a.layer * (a.m + 1);
-    for (int c = threadIdx.x; c <= a.m; c += blockDim.x) s_phase[c] = ph[c];
-  }
-  __syncthreads();
 }
 
 // Sets up the per-launch tables: phase[layer][c] (times the previous layer's
@@ -275,37 +200,32 @@ __device__ __forceinline__ void rx_round(T* tile, uint32_t tsize, int b, R r) {
   }
 }
 
+// A layer of a state smaller than a tile: one CTA, the state in shared memory.
 template <typename T>
-__global__ void __launch_bounds__(kSvThreads) sv_pass_kernel(const SvArgs a) {
+__global__ void __launch_bounds__(kSvThreads) sv_small_kernel(const SvArgs a) {
   using R = typename RealOf<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tile = reinterpret_cast<T*>(smem_raw);
   __shared__ T s_phase[kSvMaxEdges + 1];
-  __shared__ SvBlock s_sb;
   __shared__ double s_red[kSvThreads / 32];
-  const int n = a.n;
-  const bool pass0 = a.lo == 0;
-  const int rl = a.rl;
-  const int tb = pass0 ? a.len : rl + a.len;
+  const int n = a.n, tb = n;
   const uint32_t tsize = 1u << tb;
-  const uint64_t blk = blockIdx.x;
-  auto gidx = [&](uint32_t t) -> uint64_t { return sv_gidx<T>(a, blk, t); };
-  sv_block_setup<T>(a, blk, tb, s_sb, s_phase);
+  const T* phase = reinterpret_cast<const T*>(a.phase) + (size_t)a.layer * (a.m + 1);
+  for (int c = threadIdx.x; c <= a.m; c += blockDim.x) s_phase[c] = phase[c];
+  __syncthreads();
   const T rot = reinterpret_cast<const T*>(a.rot)[a.layer];
   const R rr = rot.x;
   const bool kc = rot.y != (R)0;
-  auto cut = [&](uint32_t t) -> int {
-    return s_sb.c0 + s_sb.lo[t & 127u] + s_sb.hi[t >> 7] + (int)__ldg(a.wcut + t);
-  };
+  auto cut = [&](uint32_t t) { return (int)__ldg(a.wcut + t); };
   T* psi = reinterpret_cast<T*>(a.psi);
   const R amp0 = (R)exp2(-0.5 * n);
 
   // Load.  With at least one element per thread, lanes hold consecutive tile
-  // elements (coalesced loads, conflict-free stores) and pass 0 mixes tile
-  // qubits 0..4 with shuffles (the partner of lane l for qubit q is l ^ 2^q:
+  // elements (coalesced loads, conflict-free stores) and qubits 0..4 are
+  // mixed with shuffles (the partner of lane l for qubit q is l ^ 2^q:
   // x' = c x - i s partner, the same on both sides of the pair).
   const bool full_warps = tsize >= (uint32_t)blockDim.x;
-  const int shuffled = pass0 && full_warps ? (tb < 5 ? tb : 5) : 0;
+  const int shuffled = full_warps ? (tb < 5 ? tb : 5) : 0;
   constexpr int kBatch = 8;
   for (uint32_t t0 = 0; t0 < tsize; t0 += kBatch * blockDim.x) {
     T v[kBatch];
@@ -313,18 +233,18 @@ __global__ void __launch_bounds__(kSvThreads) sv_pass_kernel(const SvArgs a) {
     for (int k = 0; k < kBatch; ++k) {
       const uint32_t t = t0 + k * blockDim.x + threadIdx.x;
       if (t < tsize) {
-        if (pass0 && a.first) {
+        if (a.first) {
           v[k].x = amp0;
           v[k].y = 0;
         } else {
-          v[k] = psi[gidx(t)];
+          v[k] = psi[t];
         }
       }
     }
 #pragma unroll
     for (int k = 0; k < kBatch; ++k) {
       const uint32_t t = t0 + k * blockDim.x + threadIdx.x;
-      if (pass0 && t < tsize) {
+      if (t < tsize) {
         const T ph = s_phase[cut(t)];
         const T x = v[k];
         v[k].x = x.x * ph.x - x.y * ph.y;
@@ -338,8 +258,8 @@ __global__ void __launch_bounds__(kSvThreads) sv_pass_kernel(const SvArgs a) {
       if (t < tsize) tile[t] = v[k];
     }
   }
-  // the remaining qubits of the pass, three at a time
-  for (int b = pass0 ? shuffled : rl; b < tb; b += 3) {
+  // the remaining qubits, three at a time
+  for (int b = shuffled; b < tb; b += 3) {
     __syncthreads();
     const int k = tb - b < 3 ? tb - b : 3;
     if (kc) {
@@ -362,7 +282,7 @@ __global__ void __launch_bounds__(kSvThreads) sv_pass_kernel(const SvArgs a) {
       v.x *= fin;
       v.y *= fin;
     }
-    if (a.store) psi[gidx(t)] = v;
+    if (a.store) psi[t] = v;
   }
   if (!a.last) return;
   for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
@@ -375,119 +295,119 @@ __global__ void __launch_bounds__(kSvThreads) sv_pass_kernel(const SvArgs a) {
   }
 }
 
-// A full tile (2^tb elements, tb = sv_tile_bits) with 2^K elements per
-// thread held in registers.  In every layout lanes are tile bits 0..4
-// (consecutive elements: coalesced global access, conflict-free shared
-// memory) and the registers are K consecutive tile bits r0..r0+K-1; the warp
-// index fills the other bits.  The load layout has the registers on the top
-// K bits, which are mixed right after the load (pass 0: after the phase);
-// mixed lane bits use shuffles; the bits in between are mixed in rounds
-// through shared memory, K at a time (one store and one load per element);
-// the pass stores from its last layout.  Bits below the pass's carried range
-// (rl, passes after the first) are not mixed.  Per layout a thread computes
-// its base tile index, global offset and linear cut term once; register r
-// adds r << r0 to the tile index, its deposit to the global offset and its
-// bits' cut coefficients.
+// A full tile of 2^(K + 8) elements with 2^K per thread in registers (K = 5 for
+// complex64, 4 for complex128; 256 threads, two CTAs per SM, so that each thread
+// has 2^K loads in flight).  Two layouts of the tile index:
+//  * top: registers on the top K bits; lanes on bits 0..4, except that the last
+//    `sh` (at most two) lane bits take tile bits 8 - sh .. 7 when these are the
+//    only mixed bits below the registers: they are mixed by shuffles, and the
+//    pass needs no shared memory;
+//  * low: registers on bits 8 - K .. 7, lanes on the bits below and the first
+//    ones above, reached by one exchange through shared memory (pass 0, and
+//    passes that mix more than two bits below the top ones).
+// The mixer's shuffles and shared-memory round trips share one pipe, which bounds
+// passes that compute cut(x): per amplitude pass 0 took ten shuffles, a table
+// lookup and an exchange with 16 elements per thread; with 32 it takes six and an
+// exchange (p=1 n=26 complex64 675 -> 508 us; p=3 n=21 149 -> 119 us).  cut(x) of a thread's elements comes from the adjacency masks by bit
+// counts: cut(x | r) = cut(x) + sum_{k in r} c_k - 2 e(r), c_k = degree of
+// register bit k's vertex - 2 popc(its neighbours in x), e(r) the edges among the
+// register bits of r (one table per CTA).
+constexpr int kSvWideThreads = 256;
+
 template <int K, bool KC, typename T, typename R>
-__device__ __forceinline__ void rx_reg_bits(T (&v)[1 << K], int r0, int lo, int hi, R r) {
+__device__ __forceinline__ void rx_reg_bits(T (&v)[1 << K], int r0, int lo, R r) {
 #pragma unroll
   for (int q = 0; q < K; ++q)
-    if (r0 + q >= lo && r0 + q < hi)
+    if (r0 + q >= lo)
 #pragma unroll
       for (int i = 0; i < (1 << K); ++i)
         if (!((i >> q) & 1)) rxs_pair<KC>(v[i], v[i | (1 << q)], r);
 }
 
-template <typename T, int K>
-__global__ void __launch_bounds__(kSvThreads, 2) sv_tile_kernel(const SvArgs a) {
+// Register r's part of an index whose register bits have the offsets g.
+template <int K>
+__device__ __forceinline__ uint32_t reg_offset(const uint32_t (&g)[K], int r) {
+  uint32_t o = 0;
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    if ((r >> k) & 1) o |= g[k];
+  return o;
+}
+
+template <typename T, int K, bool pass0>
+__global__ void __launch_bounds__(kSvWideThreads, 2) sv_wide_kernel(const SvArgs a) {
   using R = typename RealOf<T>::type;
-  constexpr int NR = 1 << K;
+  constexpr int NR = 1 << K, TB = K + 8, NB = 8 - K;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tile = reinterpret_cast<T*>(smem_raw);
   __shared__ T s_phase[kSvMaxEdges + 1];
   __shared__ uint32_t s_adj[32];
-  __shared__ int s_coef[16];
-  __shared__ int s_c0;
-  __shared__ double s_red[kSvThreads / 32];
-  const int n = a.n;
-  const bool pass0 = a.lo == 0;
-  const int tb = pass0 ? a.len : a.rl + a.len;   // K + 9 (512 threads)
-  const int mix_lo = pass0 ? 0 : a.rl;           // lowest mixed tile bit
-  const uint64_t n_tiles = 1ull << (n - tb);
-  const bool need_cut = a.wcut != nullptr;       // pass 0 and the last pass
-  // once per CTA: adjacency masks, the layer's phase table, the rotation
+  __shared__ int s_inner[2][NR];   // -2 e(r) of the top and of the low layout
+  __shared__ double s_red[kSvWideThreads / 32];
+  const int n = a.n, rl = a.rl, lo = a.lo;
+  const int mix_lo = pass0 ? 0 : rl;
+  const int below = mix_lo < 8 ? 8 - mix_lo : 0;   // mixed bits below the top registers
+  const bool exchange = pass0 || below > 2;
+  const int sh = exchange ? 0 : below;
+  const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
+  auto vertex = [&](int j) { return pass0 || j < rl ? j : lo + j - rl; };
+  // tile index of a thread (registers zero) in each layout, register offsets
+  const uint32_t top_base = (lane & ((1u << (5 - sh)) - 1u)) | (w << (5 - sh)) |
+                            ((lane >> (5 - sh)) << (8 - sh));
+  const uint32_t low_base = (lane & ((1u << NB) - 1u)) |
+                            (((lane >> NB) | (w << (5 - NB))) << 8);
+  uint32_t g_top[K], g_low[K];
   if (threadIdx.x < 32) s_adj[threadIdx.x] = (int)threadIdx.x < n ? a.adj[threadIdx.x] : 0u;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    g_top[k] = 1u << vertex(8 + k);
+    g_low[k] = 1u << vertex(NB + k);
+  }
+  if (threadIdx.x < 2 * NR) {
+    const int r = threadIdx.x & (NR - 1);
+    const bool low = threadIdx.x >= NR;
+    const uint32_t o = low ? reg_offset<K>(g_low, r) : reg_offset<K>(g_top, r);
+    int e = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if ((r >> k) & 1) e += __popc(s_adj[vertex((low ? NB : 8) + k)] & o);
+    s_inner[low][r] = -e;          // each inner edge counted from both ends: 2 e(r)
+  }
   if (pass0) {
     const T* ph = reinterpret_cast<const T*>(a.phase) + (size_t)a.layer * (a.m + 1);
-    for (int c = threadIdx.x; c <= a.m; c += blockDim.x) s_phase[c] = ph[c];
+    for (int c = threadIdx.x; c <= a.m; c += kSvWideThreads) s_phase[c] = ph[c];
   }
   const T rot = reinterpret_cast<const T*>(a.rot)[a.layer];
   const R rr = rot.x;
   const bool kc = rot.y != (R)0;   // the form of the layer's rotation (uniform)
-  const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
-  const uint32_t full = n == 32 ? 0xFFFFFFFFu : ((1u << n) - 1u);
-  const uint32_t tmask = pass0 ? (uint32_t)((1u << tb) - 1u)
-                               : (((1u << a.rl) - 1u) | (((1u << a.len) - 1u) << a.lo));
-  const uint32_t low_mask = pass0 ? 0xFFFFFFFFu : ((1u << a.rl) - 1u);
-  auto gbits = [&](uint32_t tbits) -> uint64_t {   // tile bits -> global bits
-    return pass0 ? (uint64_t)tbits
-                 : ((uint64_t)(tbits & low_mask) | ((uint64_t)(tbits >> a.rl) << a.lo));
-  };
   T* psi = reinterpret_cast<T*>(a.psi);
+  const R fin = a.last ? (R)a.scale->x : (R)1;
   R part = 0;
   __syncthreads();
-  for (uint64_t blk = blockIdx.x; blk < n_tiles; blk += gridDim.x) {
-    if (need_cut) {
-      // this tile's cut terms from its fixed bits f (see the file comment)
-      const uint32_t fm = full & ~tmask;
-      const uint32_t f = (uint32_t)sv_gidx<T>(a, blk, 0);
-      __syncthreads();   // the previous tile's readers of s_c0 / s_coef are done
-      if (threadIdx.x < 32) {
-        int c = 0;
-        const int v = threadIdx.x;
-        if (v < n) {
-          const uint32_t adj_f = s_adj[v] & fm;
-          if ((tmask >> v) & 1u) c = __popc(adj_f & f);
-          else if ((f >> v) & 1u) c = __popc(adj_f & ~f);
-        }
-        for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
-        if (v == 0) s_c0 = c;
-      }
-      if (threadIdx.x < (unsigned)tb) {
-        const int j = threadIdx.x;
-        const int v = pass0 || j < a.rl ? j : a.lo + j - a.rl;
-        const uint32_t adj_f = s_adj[v] & fm;
-        s_coef[j] = __popc(adj_f) - 2 * __popc(adj_f & f);
-      }
-      __syncthreads();
-    }
-    // register bits r0..r0+K-1 of a layout: tile index, global offset, linear
-    // cut term and the registers' cut coefficients
-    uint32_t tbase = 0;
-    uint64_t gbase = 0;
-    int lin = 0, cr[K];
-    auto set_layout = [&](int r0) {
-      const uint32_t wl = w & ((1u << (r0 - 5)) - 1u), wh = w >> (r0 - 5);
-      tbase = lane | (wl << 5) | (wh << (r0 + K));
-      gbase = sv_gidx<T>(a, blk, tbase);
-      if (need_cut) {
-        lin = s_c0;
-        for (int j = 0; j < tb; ++j)
-          if ((tbase >> j) & 1u) lin += s_coef[j];
+  // f(r, cut) for the registers of a layout (first register bit j0), x their index
+  // with registers zero; registers in Gray code order, one addition apart
+  auto each_cut = [&](uint32_t x, int j0, const int* inner, auto&& f) {
+    int c = 0, ck[K];
+    for (int q = 0; q < n; ++q) c += (x >> q) & 1u ? __popc(s_adj[q] & ~x) : 0;
 #pragma unroll
-        for (int k = 0; k < K; ++k) cr[k] = s_coef[r0 + k];
-      }
-    };
-    auto cut_of = [&](int r0, int r) -> int {
-      int c = lin;
+    for (int k = 0; k < K; ++k) {
+      const uint32_t m = s_adj[vertex(j0 + k)];
+      ck[k] = __popc(m) - 2 * __popc(m & x);
+    }
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      const int r = i ^ (i >> 1), was = i ? (i - 1) ^ ((i - 1) >> 1) : 0;
 #pragma unroll
       for (int k = 0; k < K; ++k)
-        if ((r >> k) & 1) c += cr[k];
-      return c + (int)__ldg(a.wcut + (tbase | ((uint32_t)r << r0)));
-    };
+        if (((r ^ was) >> k) & 1) c += (r >> k) & 1 ? ck[k] : -ck[k];
+      f(r, c + inner[r]);
+    }
+  };
+  const uint32_t n_tiles = (uint32_t)(1ull << (n - TB));
+  for (uint32_t blk = blockIdx.x; blk < n_tiles; blk += gridDim.x) {
+    uint32_t x = (uint32_t)sv_gidx<T>(a, blk, top_base);
     T v[NR];
-    int r0 = tb - K;
-    set_layout(r0);
     if (pass0 && a.first) {
       const R amp0 = (R)exp2(-0.5 * n);
 #pragma unroll
@@ -497,56 +417,59 @@ __global__ void __launch_bounds__(kSvThreads, 2) sv_tile_kernel(const SvArgs a) 
       }
     } else {
 #pragma unroll
-      for (int r = 0; r < NR; ++r) v[r] = psi[gbase | gbits((uint32_t)r << r0)];
+      for (int r = 0; r < NR; ++r) v[r] = psi[x | reg_offset<K>(g_top, r)];
     }
     if (pass0) {
-#pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        const T ph = s_phase[cut_of(r0, r)];
-        const T x = v[r];
-        v[r].x = x.x * ph.x - x.y * ph.y;
-        v[r].y = x.x * ph.y + x.y * ph.x;
-      }
+      each_cut(x, 8, s_inner[0], [&](int r, int c) {
+        const T ph = s_phase[c], y = v[r];
+        v[r].x = y.x * ph.x - y.y * ph.y;
+        v[r].y = y.x * ph.y + y.y * ph.x;
+      });
     }
-    if (kc) rx_reg_bits<K, true>(v, r0, mix_lo, tb, rr);
-    else rx_reg_bits<K, false>(v, r0, mix_lo, tb, rr);
-    // lane bits (tile bits 0..4) that the pass mixes: shuffles
-    for (int q = mix_lo; q < 5; ++q)
+    if (kc) rx_reg_bits<K, true>(v, 8, mix_lo, rr);
+    else rx_reg_bits<K, false>(v, 8, mix_lo, rr);
+    for (int q = 5 - sh; q < 5; ++q)
 #pragma unroll
       for (int r = 0; r < NR; ++r) {
         if (kc) rxs_shfl<true>(v[r], rr, q);
         else rxs_shfl<false>(v[r], rr, q);
       }
-    // bits 5..tb-K-1 in rounds of K through shared memory
-    for (int b = 5; b < tb - K; b += K) {
-      const int hi = min(b + K, tb - K);
-      if (hi <= mix_lo) continue;   // carried bits only
+    if (exchange) {
+      // (bit 3 flipped by bit 8: the reads of a half warp, bits 0..2 and 8, then
+      // fall into distinct banks; 16-byte elements need no flip)
+      auto at = [](uint32_t i) { return sizeof(T) == 8 ? i ^ ((i >> 5) & 8u) : i; };
       __syncthreads();   // earlier readers of the tile are done
 #pragma unroll
-      for (int r = 0; r < NR; ++r) tile[tbase | ((uint32_t)r << r0)] = v[r];
+      for (int r = 0; r < NR; ++r) tile[at(top_base | ((uint32_t)r << 8))] = v[r];
       __syncthreads();
-      r0 = min(b, tb - 2 * K);
-      set_layout(r0);
 #pragma unroll
-      for (int r = 0; r < NR; ++r) v[r] = tile[tbase | ((uint32_t)r << r0)];
-      if (kc) rx_reg_bits<K, true>(v, r0, max(b, mix_lo), hi, rr);
-      else rx_reg_bits<K, false>(v, r0, max(b, mix_lo), hi, rr);
+      for (int r = 0; r < NR; ++r) v[r] = tile[at(low_base | ((uint32_t)r << NB))];
+      x = (uint32_t)sv_gidx<T>(a, blk, low_base);
+      if (kc) rx_reg_bits<K, true>(v, NB, mix_lo, rr);
+      else rx_reg_bits<K, false>(v, NB, mix_lo, rr);
+      for (int q = mix_lo; q < NB; ++q)
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          if (kc) rxs_shfl<true>(v[r], rr, q);
+          else rxs_shfl<false>(v[r], rr, q);
+        }
     }
-    if (!a.last) {
-#pragma unroll
-      for (int r = 0; r < NR; ++r) psi[gbase | gbits((uint32_t)r << r0)] = v[r];
-      continue;
+    if (a.last) {
+      auto add = [&](int r, int c) {
+        part += (v[r].x * v[r].x + v[r].y * v[r].y) * (R)c;
+        v[r].x *= fin;
+        v[r].y *= fin;
+      };
+      if (exchange) each_cut(x, NB, s_inner[1], add);
+      else each_cut(x, 8, s_inner[0], add);
     }
-    const R fin = (R)a.scale->x;
+    if (!a.store) continue;
+    if (exchange) {
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      part += (v[r].x * v[r].x + v[r].y * v[r].y) * (R)cut_of(r0, r);
-      if (a.store) {
-        T o = v[r];
-        o.x *= fin;
-        o.y *= fin;
-        psi[gbase | gbits((uint32_t)r << r0)] = o;
-      }
+      for (int r = 0; r < NR; ++r) psi[x | reg_offset<K>(g_low, r)] = v[r];
+    } else {
+#pragma unroll
+      for (int r = 0; r < NR; ++r) psi[x | reg_offset<K>(g_top, r)] = v[r];
     }
   }
   if (!a.last) return;
@@ -555,7 +478,7 @@ __global__ void __launch_bounds__(kSvThreads, 2) sv_tile_kernel(const SvArgs a) 
   __syncthreads();
   if (threadIdx.x == 0) {
     double sum = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) sum += s_red[i];
+    for (int i = 0; i < kSvWideThreads / 32; ++i) sum += s_red[i];
     atomicAdd(&a.acc[0], sum * a.scale->y);
   }
 }
@@ -835,7 +758,7 @@ static cudaError_t sv_launch_t(void* psi, int n, int m, const uint32_t* adj_dev,
       a.rl = rl[k];
       a.first = layer == 0 && k == 0;
       a.last = layer == p - 1 && k == passes - 1;
-      a.wcut = k == 0 ? tabs.wcut_first : (a.last ? tabs.wcut_last : nullptr);
+      a.wcut = tabs.wcut;
       a.store = !(a.last && !per_edge);
       a.scale = scale;
       a.acc = acc_dev;
@@ -843,17 +766,20 @@ static cudaError_t sv_launch_t(void* psi, int n, int m, const uint32_t* adj_dev,
       const size_t smem = sizeof(T) << tb;
       const unsigned blocks = (unsigned)(1ull << (n - tb));
       if (tb == tmax) {
-        // full tiles: registers hold 2^K elements per thread (K + 9 = tb)
-        // one CTA per resident slot (two per SM), each walking tiles
-        constexpr int K = sizeof(T) == 16 ? 3 : 4;
-        cudaFuncSetAttribute(sv_tile_kernel<T, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+        // full tiles: 2^K elements per thread in registers (K + 8 = tb); one CTA per
+        // resident slot (two per SM), each walking tiles
+        constexpr int K = sizeof(T) == 16 ? 4 : 5;
         const unsigned grid = std::min<unsigned>(blocks, 2u * (unsigned)sms);
-        sv_tile_kernel<T, K><<<grid, kSvThreads, smem, stream>>>(a);
+        auto run = [&](auto kernel) {
+          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+          kernel<<<grid, kSvWideThreads, smem, stream>>>(a);
+        };
+        if (k == 0) run(sv_wide_kernel<T, K, true>);
+        else run(sv_wide_kernel<T, K, false>);
       } else {
-        cudaFuncSetAttribute(sv_pass_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(sv_small_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-        sv_pass_kernel<T><<<blocks, kSvThreads, smem, stream>>>(a);
+        sv_small_kernel<T><<<1, kSvThreads, smem, stream>>>(a);
       }
       ++*launches;
       err = cudaGetLastError();

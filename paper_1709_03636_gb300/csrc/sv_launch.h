@@ -18,14 +18,12 @@ int sv_tile_bits(int dtype);
 // 16).
 int sv_passes(int n, int tmax, int* lo, int* len, int* rl);
 
-// Cut edges inside a pass's tile for every tile index (tile bit j = vertex j,
-// or for lo > 0: bits 0..rl-1 = vertices 0..rl-1, bit rl + i = vertex lo + i).
-std::vector<uint16_t> sv_cut_table(const std::vector<uint32_t>& adj, int n, int lo, int len,
-                                   int rl);
+// cut(x) of every x of a state smaller than a tile (adj: neighbours of each qubit
+// as bit masks).
+std::vector<uint16_t> sv_cut_table(const std::vector<uint32_t>& adj);
 
 struct SvTables {
-  const uint16_t* wcut_first;   // sv_cut_table of pass 0
-  const uint16_t* wcut_last;    // sv_cut_table of the last pass (when there are several)
+  const uint16_t* wcut;         // sv_cut_table when n < sv_tile_bits, else null
   void* scratch;                // p (m + 1) + p + 2 elements of 16 bytes: phase and rotation
                                 // tables, the last layer's scale
 };

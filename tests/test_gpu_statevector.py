@@ -44,6 +44,22 @@ def test_statevector_value_only_matches_oracle(engine, n, d, p, dtype, tol):
     assert abs(C - sv.maxcut_expectation(n, edges, g, b)) < tol * len(edges)
 
 
+@pytest.mark.parametrize("n", [14, 18, 20, 21])
+@pytest.mark.parametrize("dtype,tol", [("c128", 1e-11), ("c64", 2e-6)])
+def test_statevector_every_tile_layout(engine, n, dtype, tol):
+    """Together with the sizes above: passes that mix none, one or two bits below
+    the registers' and passes that exchange, stored and only reduced."""
+    edges = [tuple(sorted(e)) for e in random_regular_graph(n, 4, n)]
+    g, b = [0.35, 1.7], [1.05, 0.5]
+    circ = q.Circuit.qaoa(n, edges, 2)
+    want = sv.maxcut_expectation(n, edges, g, b)
+    C, _ = q.statevector_expectation(engine, circ, g, b, dtype, per_edge=False)
+    assert abs(C - want) < tol * len(edges)
+    C, per_edge = q.statevector_expectation(engine, circ, g, b, dtype, per_edge=True)
+    assert abs(C - want) < tol * len(edges)
+    assert abs(0.5 * (len(edges) - sum(per_edge)) - want) < tol * len(edges)
+
+
 @pytest.mark.parametrize("n,d", [(23, 6), (26, 7)])
 @pytest.mark.parametrize("dtype,tol", [("c128", 1e-9), ("c64", 1e-5)])
 def test_statevector_value_only_p1_closed_form(n, d, dtype, tol):
