@@ -489,12 +489,14 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
     return best;
   };
   const TreeModel model = tree_model(hp.dtype);
-  // A network's steps are cut finer when few networks share the device: one p=3
-  // edge network 551 -> 456 us.  With 120 networks the finer tasks cost more than
-  // the shorter chains give (p=3 n=60 4.50 -> 4.85 ms).
-  const uint32_t teams = (uint32_t)opts.sm_count * 4;
-  lim.min_chunks = std::min(std::max(teams / (uint32_t)N, 1u), teams);
-  if (lim.min_chunks < 32) lim.min_chunks = 1;
+  // A network's steps are cut finer, towards two tasks per SM, when few networks
+  // share the device: one p=3 edge network 551 -> 380 us (four tasks per SM 411, one
+  // 370, a half 398; over nine edge networks of 32 to 60 vertices two is the best or
+  // within 3 %).  With 120 networks the finer tasks cost more than the shorter
+  // chains give (p=3 n=60 4.50 -> 4.85 ms).
+  const uint32_t tasks = (uint32_t)opts.sm_count * 2;
+  lim.min_chunks = std::min(std::max(tasks / (uint32_t)N, 1u), tasks);
+  if (lim.min_chunks < 16) lim.min_chunks = 1;
   std::vector<NetGraph> graphs(N);
   std::vector<Error> errors(N, Error{QTC_OK, ""});
   auto lower_one = [&](int i) {
