@@ -151,7 +151,8 @@ typedef struct qtc_program_info {
   int n_warp_steps;       /* warp steps over all networks (warp teams)       */
   int max_warp_steps;     /* warp steps of the longest network               */
   int n_solo_steps;       /* of the warp steps, those one op runs alone      */
-  int stage_ops;          /* ops or warp steps a team stages at a time       */
+  int stage_ops;          /* warp steps, or 16-byte units of a CTA's program,
+                             that a team stages at a time                    */
   /* graph executor: global intermediates and adjoints summed over networks,
    * as placed (tensors whose live ranges do not meet share memory) and with
    * a region of their own per tensor (what reuse saves) */

@@ -490,7 +490,7 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
   };
   const TreeModel model = tree_model(hp.dtype);
   // A network's steps are cut finer, towards two tasks per SM, when few networks
-  // share the device: one p=3 edge network 551 -> 380 us (four tasks per SM 411, one
+  // share the device: one p=3 edge network 551 -> 376 us (four tasks per SM 411, one
   // 370, a half 398; over nine edge networks of 32 to 60 vertices two is the best or
   // within 3 %).  With 120 networks the finer tasks cost more than the shorter
   // chains give (p=3 n=60 4.50 -> 4.85 ms).
