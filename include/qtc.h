@@ -426,6 +426,10 @@ qtc_status qtc_engine_set_tile_mode(qtc_engine* e, int mode);
 qtc_status qtc_selftest_tile_steps(qtc_batch* b, int dtype, int want_grad, int force_graph,
                                    int small_rank, int tile_mode, int max_bits,
                                    double* max_err, int32_t* n_checked);
+/* Host only: the order in which a team of the graph executor runs the batches of
+ * a staged long sum, on a model in which threads meet at the barriers alone.
+ * n_faults: accesses that another thread's may overtake (0 when sound). */
+qtc_status qtc_selftest_stage_schedule(int n_batches, int fold_every, int32_t* n_faults);
 
 /* Launches a one-task program whose task waits for a counter nothing ever
  * signals, so that the bounded wait expires after the engine's wait limit and

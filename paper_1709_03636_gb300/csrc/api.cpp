@@ -306,6 +306,16 @@ extern "C" qtc_status qtc_selftest_tile_steps(qtc_batch* b, int dtype, int want_
   });
 }
 
+extern "C" qtc_status qtc_selftest_stage_schedule(int n_batches, int fold_every,
+                                                  int32_t* n_faults) {
+  return guarded([&] {
+    if (!n_faults) fail(QTC_ERR_INVALID, "null argument");
+    if (n_batches < 1 || fold_every < 1)
+      fail(QTC_ERR_INVALID, "%d batches folded every %d", n_batches, fold_every);
+    *n_faults = emulate_stage_schedule((uint32_t)n_batches, (uint32_t)fold_every);
+  });
+}
+
 extern "C" qtc_status qtc_selftest_wait_timeout(qtc_engine* e, void* stream) {
   qtc_status result = QTC_OK;
   qtc_status st = guarded([&] {

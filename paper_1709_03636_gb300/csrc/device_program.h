@@ -334,6 +334,38 @@ QTC_HD inline int stage_log2_y(uint32_t footprint_elems, uint32_t elem_bytes, in
   return l >= 4 ? l : 0;
 }
 
+// The order of a staged row's batches, for all threads of its team.  Batch k's
+// offsets are in slot k & 1 of the offset table, its elements in half k & 1 of the
+// buffer: `offsets` writes this thread's part of a batch's offsets, `issue` starts
+// its copies (reading offsets that other threads wrote), `wait` ends when its own
+// copies of the batch have landed, `add` reads the elements that all threads copied,
+// `fold` may use the half of the batch just added and ends in a barrier if it does.
+// The offsets of batch k + 2 take the slot of batch k while batch k + 1 is in
+// flight: every thread has issued batch k before an earlier barrier (the one right
+// after issue(0) for k = 0, the last of iteration k - 1 else).
+#ifdef __CUDACC__
+#pragma nv_exec_check_disable
+#endif
+template <typename Offsets, typename Issue, typename Wait, typename Sync, typename Add,
+          typename Fold>
+QTC_HD inline void stage_batches(uint32_t n, Offsets&& offsets, Issue&& issue, Wait&& wait,
+                                 Sync&& sync, Add&& add, Fold&& fold) {
+  offsets(0u);
+  if (n > 1) offsets(1u);
+  sync();
+  issue(0u);
+  sync();
+  for (uint32_t k = 0; k < n; ++k) {
+    if (k + 1 < n) issue(k + 1);
+    wait(k + 1 < n ? 1u : 0u);   // batches that may still be in flight
+    if (k + 2 < n) offsets(k + 2);
+    sync();
+    add(k);
+    sync();
+    fold(k);
+  }
+}
+
 // How the four rows of a GSF_ROWS group share operands: row-counter bit 0 and
 // bit 1 map to output labels missing from A (A's element is the same for both
 // values) or from B.

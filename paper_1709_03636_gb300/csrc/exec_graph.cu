@@ -920,10 +920,13 @@ __device__ __forceinline__ void run_stage_row(const GStep& st, const T* A, const
   }
   if (tid < ea) offa[tid] = runs_offset(st.ca, row * rowlen | pa);
   if (tid < eb) offb[tid] = runs_offset(st.cb, row * rowlen | pb);
-  for (uint32_t y = tid; y < 2 * Y && y < ny; y += kGraphBlock)
-    ytab[y] = make_uint2(runs_offset(st.ya, y), runs_offset(st.yb, y));
-  team.sync();
   const uint32_t half = Y * (ea + eb);
+  auto offsets = [&](uint32_t k) {
+    for (uint32_t y = tid; y < Y; y += kGraphBlock) {
+      const uint32_t yy = k * Y + y;
+      ytab[(k & 1u) * Y + y] = make_uint2(runs_offset(st.ya, yy), runs_offset(st.yb, yy));
+    }
+  };
   auto issue = [&](uint32_t k) {
     T* dst = buf + (k & 1u) * half;
     const uint2* yt = ytab + (k & 1u) * Y;
@@ -938,21 +941,11 @@ __device__ __forceinline__ void run_stage_row(const GStep& st, const T* A, const
 #pragma unroll
   for (int u = 0; u < 8; ++u) acc[u] = czero<T>();
   const uint32_t nb = ny >> ly, fold = ny <= kYTab ? nb : kYTab >> ly;
-  issue(0);
-  for (uint32_t k = 0; k < nb; ++k) {
-    if (k + 1 < nb) {
-      issue(k + 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
-    // offsets of the batch after next, in the slots of this one's (already used)
-    if (k + 2 < nb)
-      for (uint32_t y = tid; y < Y; y += kGraphBlock) {
-        const uint32_t yy = (k + 2) * Y + y;
-        ytab[(k & 1u) * Y + y] = make_uint2(runs_offset(st.ya, yy), runs_offset(st.yb, yy));
-      }
-    team.sync();
+  auto wait = [&](uint32_t in_flight) {
+    if (in_flight) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+  };
+  auto add = [&](uint32_t k) {
     if (active) {
       const T* a = buf + (k & 1u) * half + fa;
       const T* b = buf + (k & 1u) * half + Y * ea + fb;
@@ -964,7 +957,8 @@ __device__ __forceinline__ void run_stage_row(const GStep& st, const T* A, const
         lanes ? add_batch<T, 1, 1>(a, b, ea, eb, Y, l, acc)
               : add_batch<T, 8, 1>(a, b, ea, eb, Y, 0, acc);
     }
-    team.sync();
+  };
+  auto fold_sums = [&](uint32_t k) {
     if ((k + 1) % fold == 0) {
       if (lanes) {
         // accumulator l of output c, through the batch just used
@@ -982,7 +976,8 @@ __device__ __forceinline__ void run_stage_row(const GStep& st, const T* A, const
 #pragma unroll
       for (int u = 0; u < 8; ++u) acc[u] = czero<T>();
     }
-  }
+  };
+  stage_batches(nb, offsets, issue, wait, [&] { team.sync(); }, add, fold_sums);
   if (l == 0) C[row * rowlen + c] = total;
 }
 

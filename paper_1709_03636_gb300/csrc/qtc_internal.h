@@ -247,6 +247,7 @@ size_t tile_region_bytes(const GStep& g, size_t elem);
 double emulate_tile_step(const GStep& g, uint64_t seed);
 double emulate_rows_step(const GStep& g, uint64_t seed);
 double emulate_stage_step(const GStep& g, uint64_t seed);
+int emulate_stage_schedule(uint32_t n_batches, uint32_t fold_every);
 
 // A unit is one shared-memory subtree task or one global step (its chunks);
 // its counter reaches `target` when it is complete.

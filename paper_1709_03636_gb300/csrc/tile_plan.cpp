@@ -489,4 +489,58 @@ double emulate_stage_step(const GStep& g, uint64_t seed) {
   return err;
 }
 
+// Runs stage_batches on a model of a team whose threads meet at its barriers
+// only: between two barriers any thread may be at any point.  Counts the reads of
+// a slot or half that another thread may be writing (or the writes that meet
+// another thread's reads or writes), and the reads that find another batch or
+// copies that are not known to have landed.
+int emulate_stage_schedule(uint32_t n_batches, uint32_t fold_every) {
+  struct Place {
+    uint32_t batch = ~0u;          // what it holds, of all threads, once they met
+    bool landed = true;
+    int read = -1, wrote = -1;     // interval of the last access
+  };
+  Place table[2], buffer[2];
+  int now = 0, faults = 0;         // interval: barriers so far
+  auto write = [&](Place& x, uint32_t batch, bool landed) {
+    if (x.read == now || x.wrote == now) ++faults;
+    x.wrote = now;
+    x.batch = batch;
+    x.landed = landed;
+  };
+  auto read = [&](Place& x, uint32_t batch) {
+    if (x.wrote == now || x.batch != batch || !x.landed) ++faults;
+    x.read = now;
+  };
+  uint32_t issued = 0, added = 0;
+  stage_batches(
+      n_batches, [&](uint32_t k) { write(table[k & 1u], k, true); },
+      [&](uint32_t k) {
+        read(table[k & 1u], k);
+        write(buffer[k & 1u], k, false);
+        ++issued;
+      },
+      [&](uint32_t in_flight) {
+        // (this thread's copies: the others' are known after the next barrier)
+        for (Place& x : buffer)
+          if (x.batch != ~0u && x.batch + in_flight < issued) {
+            if (!x.landed) x.wrote = now;
+            x.landed = true;
+          }
+      },
+      [&] { ++now; },
+      [&](uint32_t k) {
+        read(buffer[k & 1u], k);
+        ++added;
+      },
+      [&](uint32_t k) {
+        if ((k + 1) % fold_every) return;
+        write(buffer[k & 1u], ~0u, true);
+        ++now;
+        read(buffer[k & 1u], ~0u);
+        ++now;
+      });
+  return faults + (added != n_batches) + (issued != n_batches);
+}
+
 }  // namespace qtc
