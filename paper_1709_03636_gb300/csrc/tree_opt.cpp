@@ -40,12 +40,16 @@ struct Tree {
   }
 };
 
+// Labels of one step, at most: trees with wider steps stay as they are (they are
+// far beyond the device's memory).
+constexpr int kMaxStepLabels = 64;
+
 // Expected time (ns over the whole device) of one step, from tables over the
 // ranks of its tensors and the number of its labels.
 struct StepTimes {
-  double move[65], work[65], fixed;
+  double move[kMaxStepLabels + 1], work[kMaxStepLabels + 1], fixed;
   explicit StepTimes(const TreeModel& m) : fixed(m.step_ns) {
-    for (int i = 0; i <= 64; ++i) {
+    for (int i = 0; i <= kMaxStepLabels; ++i) {
       move[i] = m.elem * std::ldexp(1.0, i) / m.bytes_per_ns;
       work[i] = std::ldexp(1.0, i) / m.macs_per_ns;
     }
@@ -58,11 +62,17 @@ struct StepTimes {
   }
 };
 
-double step_of(Tree& t, int x, const StepTimes& time) {
+int labels_of_step(Tree& t, int x) {
   int all = 0;
   for (int w = 0; w < t.words; ++w)
     all += __builtin_popcountll(t.labels(t.left[x])[w] | t.labels(t.right[x])[w]);
-  return time(t.rank(t.left[x]), t.rank(t.right[x]), t.rank(x), all);
+  return all;
+}
+
+// (no step of a tree under search has more than kMaxStepLabels labels: the given
+// ones were looked at, the new ones hold labels of one 64-bit word)
+double step_of(Tree& t, int x, const StepTimes& time) {
+  return time(t.rank(t.left[x]), t.rank(t.right[x]), t.rank(x), labels_of_step(t, x));
 }
 
 // Rearranges the tree below `node`; true when that made it faster.
@@ -94,7 +104,7 @@ bool rearrange(Tree& t, int node, int width, const StepTimes& time, double least
     for (int i = 0; i < k; ++i) any |= t.labels(frontier[i])[w];
     for (; any; any &= any - 1) local.push_back(64 * w + __builtin_ctzll(any));
   }
-  if (local.size() > 64) return false;
+  if (local.size() > kMaxStepLabels) return false;
   auto pack = [&](int x) {
     uint64_t v = 0;
     const uint64_t* l = t.labels(x);
@@ -203,6 +213,8 @@ Plan execution_plan(const Plan& plan, const TreeModel& m) {
     t.left[L + s] = plan.steps[s].a;
     t.right[L + s] = plan.steps[s].b;
   }
+  for (int x = L; x < L + S; ++x)
+    if (labels_of_step(t, x) > kMaxStepLabels) return plan;
   const StepTimes time(m);
   std::vector<int> order;          // inner nodes, children before parents
   auto walk = [&](Tree& t) {
