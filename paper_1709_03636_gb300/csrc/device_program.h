@@ -132,10 +132,16 @@ struct alignas(16) CLane {
 };
 enum CLaneFlag : uint8_t { CLF_STORE = 4, CLF_DOT = 8 };
 static_assert(sizeof(CLane) == 16, "one unit per lane");
-// Leaf dots of lanes go to an accumulator per (parameter, lane) of the warp that
-// owns the parameter (slot modulo the team's warps), summed at the task's end;
-// programs with more parameters keep their leaf dots in SOps.
+// Leaf dots are among the first 32 lanes of their records, so that one warp, the
+// team's first, runs them all: their accumulators, one per (parameter, lane), need no
+// synchronisation between records.  At the task's end the warps share the parameters
+// and sum them.  Programs with more parameters keep their leaf dots in SOps.
 constexpr int kLaneDotSlots = 8;
+// Bytes of a graph-executor task's accumulators: FP64 in every element type, as its
+// slots are (a task sums all leaves of its subtree; in FP32 150 equal terms of 0.35 came
+// out 5e-7 off).  Dense p=2 n=100 value + gradient: 909 to 922 us, 900 with sums in
+// FP32; dots over several warps, with accumulators each, measured the same.
+QTC_HD inline uint32_t lane_dot_bytes(int n_params) { return 32u * 16u * (uint32_t)n_params; }
 constexpr uint32_t kSOpUnits = 5;
 // Units of half of a stage of `bytes` bytes (at most 8 KiB a half).
 QTC_HD inline uint32_t smem_stage_half(uint32_t bytes) {

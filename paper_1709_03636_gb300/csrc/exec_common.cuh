@@ -546,6 +546,19 @@ __device__ __forceinline__ void run_op(const SOp& op, const TeamT& team, const A
   if (flags & SOPF_SYNC) team.sync();
 }
 
+// One term of a leaf's dot into its accumulator: in the element type (as the
+// networks that run in shared memory alone keep their slots), or in FP64 (the graph
+// executor's).
+template <typename T>
+__device__ __forceinline__ void add_dot(T& sum, T v, T d) {
+  sum = cfma(v, d, sum);
+}
+__device__ __forceinline__ void add_dot(double2& sum, float2 v, float2 d) {
+  const float2 t = cfma(v, d, czero<float2>());
+  sum.x += (double)t.x;
+  sum.y += (double)t.y;
+}
+
 // A team's program (see CLane): runs the stream's batches, each copied into one
 // half of `stage` while the other half's records run.  `lacc`: accumulators of
 // lane leaf dots (n_dots parameters x 32 lanes), or null.  Every record of a
@@ -554,15 +567,16 @@ __device__ __forceinline__ void run_op(const SOp& op, const TeamT& team, const A
 // through shared memory and the barrier (an op run from its record forms its
 // offsets first, 100 instructions or so).  The p=2 n=100 gradient launch (250
 // networks of about 485 ops in 163 levels): 209 -> 115 us.
-template <typename T, int kLog, typename TeamT, typename At, typename G, typename Result>
+template <typename T, int kLog, typename TeamT, typename At, typename A, typename G,
+          typename Result>
 __device__ __forceinline__ void run_stream(const uint4* src, uint32_t units, uint4* stage,
                                            uint32_t half, const TeamT& team, const At& at,
-                                           T* table, T* lacc, int n_dots, G* grad,
+                                           T* table, A* lacc, int n_dots, G* grad,
                                            const Result& result) {
   const uint32_t tid = team.tid, lane = tid & 31u, warp = tid >> 5;
   constexpr uint32_t kWarps = 1u << (kLog - 5);
   if (lacc)
-    for (int q = (int)warp; q < n_dots; q += (int)kWarps) lacc[q * 32 + lane] = czero<T>();
+    for (int q = (int)warp; q < n_dots; q += (int)kWarps) lacc[q * 32 + lane] = czero<A>();
   for (uint32_t u = tid; u < units; u += 1u << kLog) cp_async16(stage + u, src + u);
   uint4* cur = stage;
   uint4* other = stage + half;
@@ -608,8 +622,7 @@ __device__ __forceinline__ void run_stream(const uint4* src, uint32_t units, uin
           }
           if (flags & CLF_STORE) *at(L.x & 0xffffu, 0u) = acc;
           if (flags & CLF_DOT) {
-            T* s = lacc + (L.y >> 24) * 32u + lane;
-            *s = cfma(acc, table[L.x & 0xffffu], *s);
+            add_dot(lacc[(L.y >> 24) * 32u + lane], acc, table[L.x & 0xffffu]);
           }
         }
         i += 1u << kLog;
@@ -634,7 +647,7 @@ __device__ __forceinline__ void run_stream(const uint4* src, uint32_t units, uin
   team.sync();
   if (lacc) {
     for (int q = (int)warp; q < n_dots; q += (int)kWarps) {
-      const T v = warp_csum(lacc[q * 32 + lane], 32u);
+      const A v = warp_csum(lacc[q * 32 + lane], 32u);
       if (lane == 0) {
         grad[2 * q] += (G)v.x;
         grad[2 * q + 1] += (G)v.y;

@@ -130,8 +130,8 @@ __device__ __forceinline__ void run_smem_task(const GraphProgDev& prog, uint32_t
   // [lane accumulators | arena | stage (two halves)]
   T* gbase = reinterpret_cast<T*>(prog.gbase);
   const bool dots = prog.lane_dots != 0;
-  T* lacc = dots ? reinterpret_cast<T*>(work) : nullptr;
-  T* arena = reinterpret_cast<T*>(work) + (dots ? 32 * P : 0);
+  double2* lacc = dots ? reinterpret_cast<double2*>(work) : nullptr;
+  T* arena = reinterpret_cast<T*>(work + (dots ? lane_dot_bytes(P) : 0u));
   uint4* stage = reinterpret_cast<uint4*>(arena + task.arena_elems);
   const uint32_t half = smem_stage_half((uint32_t)(work + prog.arena_bytes -
                                                    reinterpret_cast<unsigned char*>(stage)));

@@ -118,8 +118,8 @@ WaveHost assemble_wave(const std::vector<int>& nets, const std::vector<NetGraph>
                        kGraphWarps);
       const bool dots = hp.lane_dots;
       const uint32_t half = smem_stage_half(
-          hp.work_bytes - (uint32_t)(((dots ? 32u * (uint32_t)hp.n_params : 0u) + u.arena_elems) *
-                                     elem));
+          hp.work_bytes - (uint32_t)((dots ? lane_dot_bytes(hp.n_params) : 0u) +
+                                     u.arena_elems * elem));
       t.arena_elems = u.arena_elems;
       t.a = (uint32_t)w.stream.size();
       t.b = build_cta_stream(ops, half, kLaneLimit, dots, w.stream);
@@ -588,9 +588,6 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
     for (const GUnit& u : g.units) max_arena = std::max(max_arena, u.arena_elems);
   hp.max_arena = max_arena;
   auto round16 = [](size_t x) { return (uint32_t)((x + 15) & ~size_t(15)); };
-  // a subtree task keeps at least 2560 bytes beside the largest arena for its
-  // lane accumulators and its stage (other tasks stage more)
-  const size_t smem_task = 2560 + (size_t)max_arena * elem;
   const size_t chunk_task = 2 * (size_t)kYTab * sizeof(uint32_t) + 256 * elem +
                             3 * (size_t)kMaxChunkRows * sizeof(uint32_t);
   size_t tile_task = 0;
@@ -604,11 +601,28 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
         hp.tiles = true;
       }
     }
-  hp.lane_dots = hp.want_grad && hp.n_params <= kLaneDotSlots &&
-                 32 * hp.n_params * elem <= 2560 - 512;
-  hp.work_bytes = round16(std::max({smem_task, chunk_task, tile_task}));
   hp.table_bytes = round16((size_t)hp.table_elems * elem);
-  hp.smem = hp.table_bytes + (size_t)(hp.tensor_cores ? 4 : 1) * hp.work_bytes;
+  // A subtree task keeps at least 2560 bytes beside the largest arena for its stage, or
+  // its lane accumulators of leaf dots and 1536 (else 512) for its stage, as long as
+  // they cost no CTA per SM (other tasks stage more).  With 512 bytes, batches of 15
+  // units, the whole-network tasks of dense p=2 n=100 took long enough for 1080 us in
+  // all (920 with 1536).
+  auto layout = [&](size_t beside) {
+    hp.work_bytes =
+        round16(std::max({beside + (size_t)max_arena * elem, chunk_task, tile_task}));
+    hp.smem = hp.table_bytes + (size_t)(hp.tensor_cores ? 4 : 1) * hp.work_bytes;
+    // CTAs per SM by shared memory (228 KB; 1 KB and 3.7 KB static a CTA)
+    return hp.tensor_cores ? (hp.smem <= max_dynamic) : 233472 / (hp.smem + 4864);
+  };
+  const size_t resident = layout(2560);
+  hp.lane_dots = false;
+  if (hp.want_grad && hp.n_params <= kLaneDotSlots)
+    for (size_t stage : {1536, 512}) {
+      if (hp.lane_dots) break;
+      hp.lane_dots = layout(lane_dot_bytes(hp.n_params) + stage) >= resident &&
+                     hp.smem <= max_dynamic;
+    }
+  if (!hp.lane_dots) layout(2560);
   for (auto& wnets : waves) {
     std::sort(wnets.begin(), wnets.end());
     hp.waves.push_back(assemble_wave(wnets, graphs, elem, opts.sm_count * 4, hp));
