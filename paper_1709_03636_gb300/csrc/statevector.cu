@@ -494,125 +494,90 @@ __global__ void __launch_bounds__(kSvWideThreads, 2) sv_wide_kernel(const SvArgs
 // the last time here; the state is internal), and a second launch adds them up
 // per edge.
 //
-// GB300's FP64 pipe does two operations per clock and SM, and that is what
-// bound the former form (16 FP64 sums per amplitude and launch, m / 16
-// launches): n = 21 with 63 edges, depth 3, 654 -> 150 us in all.  complex64
-// states are summed as pairs of floats (exact products and error-free
-// additions, about 48 bits; the values agree to every float32 bit) on the FP32
-// pipe instead; complex128 in FP64, about ten operations per amplitude for all
-// edges.
+// Probabilities and sums are FP64 for both element types.  GB300's FP64 pipe does two
+// operations per clock and SM, and that bounds the kernel at about ten operations per
+// amplitude for all edges (it bound the former one at sixteen per amplitude and launch,
+// m / 16 launches): n = 21 with 63 edges, depth 3, 654 -> 150 us in all.  (Sums in pairs
+// of floats took 113 us, but held 48 bits: 1e-16 rms off the FP64 sums of the same
+// state, twice to four times what FP64 is.)
 constexpr int kZzBits = 12, kZzThreads = 256;
 
-struct FloatPair {
-  float h, l;
-};
-__device__ __forceinline__ FloatPair pair_sum(float a, float al, float b, float bl) {
-  const float s = a + b, t = s - a;
-  const float e = ((a - (s - t)) + (b - t)) + (al + bl);
-  const float h = s + e;
-  return {h, e - (h - s)};
-}
-__device__ __forceinline__ FloatPair zadd(FloatPair a, FloatPair b) {
-  return pair_sum(a.h, a.l, b.h, b.l);
-}
-__device__ __forceinline__ FloatPair zsub(FloatPair a, FloatPair b) {
-  return pair_sum(a.h, a.l, -b.h, -b.l);
-}
-__device__ __forceinline__ double zadd(double a, double b) { return a + b; }
-__device__ __forceinline__ double zsub(double a, double b) { return a - b; }
-__device__ __forceinline__ FloatPair zprob(float2 v) {
-  const float x = v.x * v.x, y = v.y * v.y;
-  return pair_sum(x, fmaf(v.x, v.x, -x), y, fmaf(v.y, v.y, -y));
-}
 __device__ __forceinline__ double zprob(double2 v) { return v.x * v.x + v.y * v.y; }
-__device__ __forceinline__ FloatPair zshfl(FloatPair v, int m) {
-  return {__shfl_xor_sync(0xffffffffu, v.h, m), __shfl_xor_sync(0xffffffffu, v.l, m)};
-}
-__device__ __forceinline__ double zshfl(double v, int m) {
-  return __shfl_xor_sync(0xffffffffu, v, m);
-}
-__device__ __forceinline__ double zdouble(FloatPair v) { return (double)v.h + (double)v.l; }
-__device__ __forceinline__ double zdouble(double v) { return v; }
-
-template <typename T> struct ZzOf;
-template <> struct ZzOf<float2> { using type = FloatPair; };
-template <> struct ZzOf<double2> { using type = double; };
 
 template <typename T>
 __global__ void __launch_bounds__(kZzThreads) sv_zz_kernel(T* psi, int n, int m, const int2* edges,
                                                            double* acc) {
-  using S = typename ZzOf<T>::type;
   // sums over subsets of register bits: none, {i}, {i, j} (i < j)
   constexpr int kSums = 11;
   __shared__ double s_sum[kSums][kZzThreads];
   __shared__ double s_warp[kZzThreads / 32][10];
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   const uint64_t n_tiles = 1ull << (n - kZzBits);
-  S total[kSums];
+  double total[kSums];
 #pragma unroll
-  for (int k = 0; k < kSums; ++k) total[k] = S{};
+  for (int k = 0; k < kSums; ++k) total[k] = 0.0;
   for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     T* at = psi + (tile << kZzBits);
-    S p[16];
+    double p[16];
     {
       T v[16];
 #pragma unroll
       for (int r = 0; r < 16; ++r) v[r] = at[(warp << 9) | (r << 5) | lane];
 #pragma unroll
-      for (int r = 0; r < 16; ++r) p[r] = zprob(v[r]);
+      for (int r = 0; r < 16; ++r) p[r] = zprob(to_d2(v[r]));
     }
     // one[i] = sum of p signed by register bit i, two[] by pairs of bits; each
     // step folds the lowest remaining bit away
-    S one[4], two[6];
+    double one[4], two[6];
     int k2 = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int half = 8 >> i;
-      S d[8];
+      double d[8];
 #pragma unroll
       for (int r = 0; r < half; ++r) {
-        d[r] = zsub(p[2 * r], p[2 * r + 1]);
-        p[r] = zadd(p[2 * r], p[2 * r + 1]);
+        d[r] = p[2 * r] - p[2 * r + 1];
+        p[r] = p[2 * r] + p[2 * r + 1];
       }
       // the differences folded further: signed by bit i and by one later bit
       int rest = half;
 #pragma unroll
       for (int j = i + 1; j < 4; ++j) {
-        S t = zsub(d[0], d[1]);
+        double t = d[0] - d[1];
 #pragma unroll
         for (int r = 1; r < 4; ++r)
-          if (2 * r < rest) t = zadd(t, zsub(d[2 * r], d[2 * r + 1]));
+          if (2 * r < rest) t += d[2 * r] - d[2 * r + 1];
         two[k2++] = t;
 #pragma unroll
         for (int r = 0; r < 4; ++r)
-          if (2 * r < rest) d[r] = zadd(d[2 * r], d[2 * r + 1]);
+          if (2 * r < rest) d[r] = d[2 * r] + d[2 * r + 1];
         rest >>= 1;
       }
       one[i] = d[0];
     }
-    total[0] = zadd(total[0], p[0]);
+    total[0] += p[0];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) total[1 + i] = zadd(total[1 + i], one[i]);
+    for (int i = 0; i < 4; ++i) total[1 + i] += one[i];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) total[5 + k] = zadd(total[5 + k], two[k]);
+    for (int k = 0; k < 6; ++k) total[5 + k] += two[k];
     // the tile's one-bit sums and total (only edges above the tile bits use
     // them): p[0] over the lanes as a Walsh-Hadamard transform, lane l ending
     // with the sum signed by subset l of the lane bits
     if (n > kZzBits) {
-      S w = p[0];
+      double w = p[0];
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
-        const S o = zshfl(w, 1 << q);
-        w = ((lane >> q) & 1u) ? zsub(o, w) : zadd(w, o);
+        const double o = __shfl_xor_sync(0xffffffffu, w, 1 << q);
+        w = ((lane >> q) & 1u) ? o - w : w + o;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) one[i] = zadd(one[i], zshfl(one[i], 1 << q));
+        for (int i = 0; i < 4; ++i) one[i] += __shfl_xor_sync(0xffffffffu, one[i], 1 << q);
       }
       const int slot = lane == 0 ? 0 : (lane & (lane - 1)) == 0 ? 32 - __clz(lane) : -1;
       __syncthreads();   // every thread has read the tile; s_warp is free
-      if (slot >= 0) s_warp[warp][slot] = zdouble(w);   // total, lane bits 0..4
+      if (slot >= 0) s_warp[warp][slot] = w;   // total, lane bits 0..4
       if (lane < 4) {
-        const S o = lane == 0 ? one[0] : lane == 1 ? one[1] : lane == 2 ? one[2] : one[3];
-        s_warp[warp][6 + lane] = zdouble(o);
+        const double o = lane == 0 ? one[0] : lane == 1 ? one[1] : lane == 2 ? one[2] : one[3];
+        s_warp[warp][6 + lane] = o;
       }
       __syncthreads();
       if (threadIdx.x < 13) {
@@ -629,7 +594,7 @@ __global__ void __launch_bounds__(kZzThreads) sv_zz_kernel(T* psi, int n, int m,
   }
   // edges inside the tile bits
 #pragma unroll
-  for (int k = 0; k < kSums; ++k) s_sum[k][threadIdx.x] = zdouble(total[k]);
+  for (int k = 0; k < kSums; ++k) s_sum[k][threadIdx.x] = total[k];
   __syncthreads();
   for (int e = warp; e < m; e += kZzThreads / 32) {
     const int2 ed = edges[e];
