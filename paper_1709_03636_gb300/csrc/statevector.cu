@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(kSvWideThreads, 2) sv_wide_kernel(const SvArgs
   __shared__ T s_phase[kSvMaxEdges + 1];
   __shared__ uint32_t s_adj[32];
   __shared__ int s_inner[2][NR];   // -2 e(r) of the top and of the low layout
-  __shared__ double s_red[kSvWideThreads / 32];
+  __shared__ double s_red[2 * kSvWideThreads / 32];
   const int n = a.n, rl = a.rl, lo = a.lo;
   const int mix_lo = pass0 ? 0 : rl;
   const int below = mix_lo < 8 ? 8 - mix_lo : 0;   // mixed bits below the top registers
@@ -381,7 +381,9 @@ __global__ void __launch_bounds__(kSvWideThreads, 2) sv_wide_kernel(const SvArgs
   const bool kc = rot.y != (R)0;   // the form of the layer's rotation (uniform)
   T* psi = reinterpret_cast<T*>(a.psi);
   const R fin = a.last ? (R)a.scale->x : (R)1;
-  R part = 0;
+  // <C>: two sums per thread, of one half of its registers each, so that a chain of
+  // single-precision additions is 16 terms per tile (complex64)
+  R part[2] = {0, 0};
   __syncthreads();
   // f(r, cut) for the registers of a layout (first register bit j0), x their index
   // with registers zero; registers in Gray code order, one addition apart
@@ -454,7 +456,7 @@ __global__ void __launch_bounds__(kSvWideThreads, 2) sv_wide_kernel(const SvArgs
     }
     if (a.last) {
       auto add = [&](int r, int c) {
-        part += (v[r].x * v[r].x + v[r].y * v[r].y) * (R)c;
+        part[r >> (K - 1)] += (v[r].x * v[r].x + v[r].y * v[r].y) * (R)c;
         v[r].x *= fin;
         v[r].y *= fin;
       };
@@ -471,12 +473,15 @@ __global__ void __launch_bounds__(kSvWideThreads, 2) sv_wide_kernel(const SvArgs
     }
   }
   if (!a.last) return;
-  for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-  if (lane == 0) s_red[w] = (double)part;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    for (int off = 16; off > 0; off >>= 1) part[h] += __shfl_xor_sync(0xffffffffu, part[h], off);
+    if (lane == 0) s_red[2 * w + h] = (double)part[h];
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     double sum = 0.0;
-    for (int i = 0; i < kSvWideThreads / 32; ++i) sum += s_red[i];
+    for (int i = 0; i < 2 * kSvWideThreads / 32; ++i) sum += s_red[i];
     atomicAdd(&a.acc[0], sum * a.scale->y);
   }
 }
