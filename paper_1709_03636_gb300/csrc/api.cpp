@@ -53,12 +53,19 @@ struct Prepared {
 
 using namespace qtc;
 
+// A number that no engine state of the process has had: programs name the state
+// whose arena they lie in by it (an engine's address may come back after its end).
+static uint64_t next_generation() {
+  static std::atomic<uint64_t> last{0};
+  return ++last;
+}
+
 struct qtc_engine {
   int device = 0;
   char* arena = nullptr;
   size_t bytes = 0;
   size_t used = 0;
-  uint64_t generation = 1;
+  uint64_t generation = next_generation();
   int sm_count = 0;
   size_t smem_optin = 0;
   int last_launches = 0;
@@ -211,7 +218,7 @@ extern "C" qtc_status qtc_engine_reset(qtc_engine* e) {
     if (!e) fail(QTC_ERR_INVALID, "null engine");
     e->used = 0;
     e->work = 0;
-    e->generation += 1;
+    e->generation = next_generation();
   });
 }
 
@@ -225,7 +232,7 @@ extern "C" qtc_status qtc_engine_set_limits(qtc_engine* e, size_t max_wave_bytes
     if (!(wait_limit_ms > 0.0)) fail(QTC_ERR_INVALID, "wait limit must be positive");
     e->options.wave_cap_bytes = max_wave_bytes;
     e->wait_limit_ms = wait_limit_ms;
-    e->generation += 1;  // programs are re-prepared with the new limits
+    e->generation = next_generation();  // programs are re-prepared with the new limits
     e->used = 0;
     e->work = 0;
   });
@@ -238,7 +245,7 @@ extern "C" qtc_status qtc_engine_set_graph_options(qtc_engine* e, int force_grap
     if (small_rank < 0 || small_rank > 16) fail(QTC_ERR_INVALID, "small rank %d", small_rank);
     e->options.force_graph = force_graph != 0;
     e->options.small_rank = small_rank;
-    e->generation += 1;
+    e->generation = next_generation();
     e->used = 0;
     e->work = 0;
   });
@@ -259,7 +266,7 @@ extern "C" qtc_status qtc_engine_set_task_options(qtc_engine* e, int task_terms_
       fail(QTC_ERR_INVALID, "warp_teams %d (0..2)", warp_teams);
     e->options.warp_teams = warp_teams;
     e->options.graph_hi_occupancy = graph_hi_occupancy != 0;
-    e->generation += 1;
+    e->generation = next_generation();
     e->used = 0;
     e->work = 0;
   });
@@ -270,7 +277,7 @@ extern "C" qtc_status qtc_engine_set_tile_mode(qtc_engine* e, int mode) {
     if (!e) fail(QTC_ERR_INVALID, "null engine");
     if (mode < 0 || mode > 4) fail(QTC_ERR_INVALID, "tile mode %d (0..4)", mode);
     e->options.tile_mode = mode;
-    e->generation += 1;
+    e->generation = next_generation();
     e->used = 0;
     e->work = 0;
   });
