@@ -1085,14 +1085,18 @@ const HostProgram& qtc::host_program(qtc_batch* b, int dtype, int want_grad,
     }
     hp->ops.clear();
     for (const auto& p : progs) hp->ops.insert(hp->ops.end(), p.begin(), p.end());
-    // lanes take more memory than records for the wider ops: not where that
-    // could outgrow an arena (or the static scratch array) that held the ops
-    for (uint32_t limit : {kLaneLimit, kLaneLimitSmall}) {
+    // lanes take more memory than records for the wider ops: not where that makes a large
+    // program larger than its ops
+    for (const bool smallest : {false, true}) {
+      if (opts.compact && !smallest) continue;
       hp->stream.clear();
       for (size_t i = 0; i < progs.size(); ++i) {
         TaskDev& t = hp->tasks[i];
         t.op_begin = (uint32_t)hp->stream.size();
-        t.op_count = build_cta_stream(progs[i], hp->half_units, limit, hp->lane_dots, hp->stream);
+        t.op_count = smallest ? build_smallest_stream(progs[i], hp->half_units, hp->lane_dots,
+                                                      hp->stream)
+                              : build_cta_stream(progs[i], hp->half_units, kLaneLimit,
+                                                 hp->lane_dots, hp->stream);
         validate_cta_stream(hp->stream.data() + t.op_begin, hp->stream.size() - t.op_begin,
                             t.op_count, hp->half_units, table_elems, t.arena_elems, P);
       }
@@ -1196,29 +1200,10 @@ static Prepared& prepare_graph(qtc_engine* e, qtc_batch* b, const HostProgram& h
   return b->prepared.back();
 }
 
-static Prepared& prepare(qtc_engine* e, qtc_batch* b, int dtype, int want_grad,
-                         cudaStream_t stream) {
-  want_grad = want_grad ? 1 : 0;
-  for (Prepared& p : b->prepared)
-    if (p.engine == e && p.generation == e->generation && p.dtype == dtype &&
-        p.want_grad == want_grad)
-      return p;
-  const size_t max_dyn = max_dynamic_smem(e->smem_optin);
-  const HostProgram& hp = host_program(b, dtype, want_grad, max_dyn, e->options);
-  if (hp.graph) {
-    const size_t used = e->used, work = e->work;
-    try {
-      return prepare_graph(e, b, hp, stream, max_dyn);
-    } catch (const Error& err) {
-      // an arena sized for the plans' own trees: contract those
-      if (err.status != QTC_ERR_ARENA) throw;
-      e->used = used;
-      e->work = work;
-    }
-    ProgramOptions own = e->options;
-    own.plan_trees = true;
-    return prepare_graph(e, b, host_program(b, dtype, want_grad, max_dyn, own), stream, max_dyn);
-  }
+// Uploads a shared-memory program.
+static Prepared& prepare_shared(qtc_engine* e, qtc_batch* b, const HostProgram& hp,
+                                cudaStream_t stream, size_t max_dyn) {
+  const int dtype = hp.dtype, want_grad = hp.want_grad;
   const int P = hp.n_params;
   const int N = hp.n_nets;
   const int G = (int)hp.gates.size();
@@ -1297,6 +1282,39 @@ static Prepared& prepare(qtc_engine* e, qtc_batch* b, int dtype, int want_grad,
   pr.per_sm = per_sm;
   b->prepared.push_back(pr);
   return b->prepared.back();
+}
+
+static Prepared& prepare(qtc_engine* e, qtc_batch* b, int dtype, int want_grad,
+                         cudaStream_t stream) {
+  want_grad = want_grad ? 1 : 0;
+  for (Prepared& p : b->prepared)
+    if (p.engine == e && p.generation == e->generation && p.dtype == dtype &&
+        p.want_grad == want_grad)
+      return p;
+  const size_t max_dyn = max_dynamic_smem(e->smem_optin);
+  auto upload = [&](const HostProgram& hp) -> Prepared& {
+    const size_t used = e->used, work = e->work;
+    try {
+      return hp.graph ? prepare_graph(e, b, hp, stream, max_dyn)
+                      : prepare_shared(e, b, hp, stream, max_dyn);
+    } catch (const Error&) {
+      e->used = used;
+      e->work = work;
+      throw;
+    }
+  };
+  const HostProgram& hp = host_program(b, dtype, want_grad, max_dyn, e->options);
+  try {
+    return upload(hp);
+  } catch (const Error& err) {
+    // (warp programs have one form)
+    if (err.status != QTC_ERR_ARENA || hp.warp_teams) throw;
+  }
+  // An arena that is too small for the faster form of the program: its smallest one
+  // (dense p=2 n=100: 4.6 MB of tables instead of 7.6, value + gradient 16.2 instead of 27.4).
+  ProgramOptions small = e->options;
+  small.compact = true;
+  return upload(host_program(b, dtype, want_grad, max_dyn, small));
 }
 
 static void launch(qtc_engine* e, const Prepared& pr, const double* params_dev, double* out_dev,

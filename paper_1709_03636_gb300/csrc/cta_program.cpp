@@ -350,7 +350,7 @@ uint32_t build_cta_stream(const std::vector<SOp>& ops, uint32_t half_units, uint
   std::vector<std::pair<size_t, size_t>> batches;
   for (size_t i = 0; i < records.size();) {
     size_t j = i;
-    uint32_t units = 1;
+    uint32_t units = i ? 1 : 0;
     while (j < records.size() && units + records[j].units.size() <= half_units)
       units += (uint32_t)records[j++].units.size();
     batches.push_back({i, j});
@@ -358,35 +358,49 @@ uint32_t build_cta_stream(const std::vector<SOp>& ops, uint32_t half_units, uint
   }
   std::vector<uint32_t> sizes;
   for (const auto& b : batches) {
-    uint32_t units = 1;
+    uint32_t units = b.first ? 1 : 0;
     for (size_t k = b.first; k < b.second; ++k) units += (uint32_t)records[k].units.size();
     sizes.push_back(units);
   }
   for (size_t n = 0; n < batches.size(); ++n) {
     const auto& b = batches[n];
-    out.push_back(uint4{(uint32_t)(b.second - b.first), n + 1 < sizes.size() ? sizes[n + 1] : 0u,
-                        0, 0});
+    if (n) out.push_back(uint4{0, n + 1 < sizes.size() ? sizes[n + 1] : 0u, 0, 0});
     for (size_t k = b.first; k < b.second; ++k) {
       if (records[k].level_end && k + 1 < b.second) records[k].units[0].x |= SOPF_SYNC << 24;
       out.insert(out.end(), records[k].units.begin(), records[k].units.end());
     }
   }
-  return sizes[0];
+  return sizes[0] | (sizes.size() > 1 ? sizes[1] << 16 : 0u);
 }
 
-void validate_cta_stream(const uint4* stream, size_t n, uint32_t units, uint32_t half_units,
+uint32_t build_smallest_stream(const std::vector<SOp>& ops, uint32_t half_units, bool dots,
+                               std::vector<uint4>& out) {
+  std::vector<uint4> best;
+  uint32_t units = 0;
+  for (uint32_t limit : {4u, 2u, 0u}) {
+    std::vector<uint4> s;
+    const uint32_t first = build_cta_stream(ops, half_units, limit, dots, s);
+    if (limit < 4u && s.size() >= best.size()) continue;
+    best.swap(s);
+    units = first;
+  }
+  out.insert(out.end(), best.begin(), best.end());
+  return units;
+}
+
+void validate_cta_stream(const uint4* stream, size_t n, uint32_t batches, uint32_t half_units,
                          uint32_t table_elems, uint32_t arena_elems, int n_params) {
   auto need = [&](bool ok, const char* what) {
     if (!ok) fail(QTC_ERR_INVALID, "internal: task stream: %s", what);
   };
   const uint32_t team_elems = table_elems + arena_elems;
   size_t at = 0;
+  uint32_t units = batches & 0xffffu;
   while (units) {
     need(units <= half_units && at + units <= n, "batch beyond the stage or the stream");
-    const uint32_t next = stream[at].y;
-    size_t u = at + 1;
-    for (uint32_t r = 0; r < stream[at].x; ++r) {
-      need(u < at + units, "records beyond their batch");
+    const uint32_t next = at ? stream[at].y : batches >> 16;
+    size_t u = at ? at + 1 : at;
+    while (u < at + units) {
       if ((stream[u].x & 15u) != SOP_LANES) {
         u += kSOpUnits;   // (checked op by op before)
         continue;

@@ -118,8 +118,10 @@ constexpr int kLeafSlotByte = 15;     // (a leaf's output has at most 4 bits)
 constexpr uint32_t kNarrowMax = 128;  // outputs of a narrow op
 
 // A task's program is a stream of 16-byte units, read in batches that fit half
-// of the team's stage.  Batch: one unit (records, units of the next batch, 0, 0;
-// the last batch names 0 units), then its records.  Record: an SOp (5 units), or
+// of the team's stage.  Batch: one unit (0, units of the next batch, 0, 0; the last
+// batch names 0 units), then its records.  The first batch has no such unit (most
+// programs are one batch): the task holds its units and the next batch's << 16.
+// Record: an SOp (5 units), or
 // a lanes record: a unit (SOP_LANES | flags << 24, lanes, 0, 0) and one CLane
 // per lane, which thread `lane` of the team runs.
 struct alignas(16) CLane {
@@ -238,7 +240,7 @@ static_assert(sizeof(WStep) == 544, "WStep is staged as 34 16-byte words");
 
 struct TaskDev {
   uint32_t op_begin, op_count;     // warp teams: steps; CTA teams: first unit, units of the
-                                   // first batch
+                                   // first two batches
   uint32_t net;
   uint32_t arena_elems;
 };
@@ -475,7 +477,7 @@ struct GTask {
   uint8_t kind;
   uint8_t pad[3];
   uint32_t a;              // SMEM: first unit; CHUNK, TC: step index
-  uint32_t b;              // SMEM: units of the first batch; CHUNK: chunk index; TC: tile index
+  uint32_t b;              // SMEM: units of the first two batches; CHUNK: chunk index; TC: tile index
   uint32_t net;
   uint32_t wait_begin;     // into the wait list
   uint32_t wait_count;

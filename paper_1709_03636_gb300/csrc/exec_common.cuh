@@ -569,24 +569,25 @@ __device__ __forceinline__ void add_dot(double2& sum, float2 v, float2 d) {
 // networks of about 485 ops in 163 levels): 209 -> 115 us.
 template <typename T, int kLog, typename TeamT, typename At, typename A, typename G,
           typename Result>
-__device__ __forceinline__ void run_stream(const uint4* src, uint32_t units, uint4* stage,
+__device__ __forceinline__ void run_stream(const uint4* src, uint32_t batches, uint4* stage,
                                            uint32_t half, const TeamT& team, const At& at,
                                            T* table, A* lacc, int n_dots, G* grad,
                                            const Result& result) {
   const uint32_t tid = team.tid, lane = tid & 31u, warp = tid >> 5;
   constexpr uint32_t kWarps = 1u << (kLog - 5);
+  uint32_t units = batches & 0xffffu, next_units = batches >> 16;
   if (lacc)
     for (int q = (int)warp; q < n_dots; q += (int)kWarps) lacc[q * 32 + lane] = czero<A>();
   for (uint32_t u = tid; u < units; u += 1u << kLog) cp_async16(stage + u, src + u);
   uint4* cur = stage;
   uint4* other = stage + half;
-  while (units) {
+  for (uint32_t head_units = 0; units; head_units = 1) {
     cp_async_wait_all();
     team.sync();
-    const uint4 batch = cur[0];
+    if (head_units) next_units = cur[0].y;
     src += units;
-    for (uint32_t u = tid; u < batch.y; u += 1u << kLog) cp_async16(other + u, src + u);
-    const uint4* rec = cur + 1;
+    for (uint32_t u = tid; u < next_units; u += 1u << kLog) cp_async16(other + u, src + u);
+    const uint4* rec = cur + head_units;
     const uint4* end = cur + units;
     uint4 head = rec[0], L = make_uint4(0, 0, 0, 0);
     bool have = (head.x & 15u) == SOP_LANES && tid < head.y;
@@ -639,7 +640,7 @@ __device__ __forceinline__ void run_stream(const uint4* src, uint32_t units, uin
       }
       if (sync) team.sync();
     }
-    units = batch.y;
+    units = next_units;
     uint4* t = cur;
     cur = other;
     other = t;

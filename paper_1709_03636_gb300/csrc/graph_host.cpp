@@ -122,7 +122,8 @@ WaveHost assemble_wave(const std::vector<int>& nets, const std::vector<NetGraph>
                                      u.arena_elems * elem));
       t.arena_elems = u.arena_elems;
       t.a = (uint32_t)w.stream.size();
-      t.b = build_cta_stream(ops, half, kLaneLimit, dots, w.stream);
+      t.b = hp.options.compact ? build_smallest_stream(ops, half, dots, w.stream)
+                               : build_cta_stream(ops, half, kLaneLimit, dots, w.stream);
       validate_cta_stream(w.stream.data() + t.a, w.stream.size() - t.a, t.b, half, hp.table_elems,
                           u.arena_elems, hp.n_params);
     } else if (u.kind == GT_TC) {
@@ -253,7 +254,8 @@ void validate_wave(const WaveHost& w, uint32_t table_elems, uint32_t arena_elems
     if (t.wait_begin + t.wait_count > w.waits.size())
       fail(QTC_ERR_INVALID, "internal: wait list out of range");
     if (t.kind == GT_SMEM) {
-      if ((uint64_t)t.a + t.b > w.stream.size()) fail(QTC_ERR_INVALID, "internal: stream range");
+      if ((uint64_t)t.a + (t.b & 0xffffu) > w.stream.size())
+        fail(QTC_ERR_INVALID, "internal: stream range");
       if (t.signal != 0xFFFFFFFFu && t.signal >= w.n_counters)
         fail(QTC_ERR_INVALID, "internal: signal counter out of range");
     } else if (t.kind == GT_TC) {
@@ -496,7 +498,8 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
   // chains give (p=3 n=60 4.50 -> 4.85 ms).
   const uint32_t tasks = (uint32_t)opts.sm_count * 2;
   lim.min_chunks = std::min(std::max(tasks / (uint32_t)N, 1u), tasks);
-  if (lim.min_chunks < 16) lim.min_chunks = 1;
+  if (lim.min_chunks < 16 || opts.compact) lim.min_chunks = 1;
+  lim.stage_rows = !opts.compact;
   std::vector<NetGraph> graphs(N);
   std::vector<Error> errors(N, Error{QTC_OK, ""});
   auto lower_one = [&](int i) {
@@ -514,7 +517,7 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
     }
     NetGraph g;
     g.fits = false;
-    if (!opts.plan_trees) g = lower_network(i, execution_plan(plans[i], model));
+    if (!opts.plan_trees && !opts.compact) g = lower_network(i, execution_plan(plans[i], model));
     if (!g.fits || over(g)) {
       // the plan's own tree, where the rearranged one cannot be lowered or
       // needs more memory than a wave may take

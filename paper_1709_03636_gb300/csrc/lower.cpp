@@ -894,7 +894,8 @@ NetGraph lower_graph(const Plan& plan, const std::vector<int>& leaf_gate,
     std::string why;
     if (!encode_gstep(u.step, lc, la, lb, leaf_for_grad >= 0, lim.task_terms_log2,
                       lim.tile_mode ? 1u : lim.min_chunks,
-                      lim.tile_mode == 0 && (!in_adjoint || lim.min_chunks > 1), lim.elem, ra.global, rb.global, &why)) {
+                      lim.stage_rows && lim.tile_mode == 0 && (!in_adjoint || lim.min_chunks > 1),
+                      lim.elem, ra.global, rb.global, &why)) {
       ng.fits = false;
       ng.why = why;
       return -1;

@@ -193,15 +193,19 @@ void validate_cta_ops(const SOp* ops, size_t n, uint32_t table_elems, uint32_t a
 
 // Appends a task's scheduled ops as a stream (see CLane) for a stage of twice
 // half_units units; ops of at most lane_limit outputs become lanes, leaf dots
-// among them only with `dots`.  Returns the units of the first batch.
+// among them only with `dots`.  Returns the units of the first two batches (the second's
+// in the high 16 bits).
 uint32_t build_cta_stream(const std::vector<SOp>& ops, uint32_t half_units, uint32_t lane_limit,
                           bool dots, std::vector<uint4>& out);
+// The shortest of the streams with lanes for ops of at most 4, 2 or no outputs.
+uint32_t build_smallest_stream(const std::vector<SOp>& ops, uint32_t half_units, bool dots,
+                               std::vector<uint4>& out);
 // Host check of one task's stream (its ops already checked).
 void validate_cta_stream(const uint4* stream, size_t n, uint32_t units, uint32_t half_units,
                          uint32_t table_elems, uint32_t arena_elems, int n_params);
-// Outputs of an op that becomes lanes: up to 16 of them cost no more memory than
-// its record, on average; 4 never more (used where memory is short).
-constexpr uint32_t kLaneLimit = 16, kLaneLimitSmall = 4;
+// Outputs of an op that becomes lanes (16 of them take more memory than its record of
+// five units).
+constexpr uint32_t kLaneLimit = 16;
 
 // Lowers one plan to a shared-memory op program.  table_elems: size of the
 // gate value + derivative region that precedes the arena.  Intermediates and
@@ -232,6 +236,7 @@ struct GraphLimits {
                                      // 3 steps summing >= 3 labels, 4 every step that tiles
   size_t elem = 8;                   // bytes per element
   uint32_t min_chunks = 1;           // tasks a global step is cut into where its rows allow
+  bool stage_rows = true;            // long sums in few tasks may be staged (more tasks)
 };
 
 // Tile form of a global step (tile_plan.cpp): fills g.tile, g.n_chunks and
@@ -316,13 +321,15 @@ struct ProgramOptions {
   bool graph_hi_occupancy = false; // graph executor: the five-CTAs-per-SM instantiation
   bool plan_trees = true;          // graph executor: contract the plans' own trees; false
                                    // (what engines run): execution_plan's
+  bool compact = false;            // the smallest program tables (implies plan_trees): few lanes
+                                   // in the streams, no steps cut finer for few networks
   bool operator==(const ProgramOptions& o) const {
     return wave_cap_bytes == o.wave_cap_bytes && force_graph == o.force_graph &&
            small_rank == o.small_rank && task_terms_log2 == o.task_terms_log2 &&
            tile_mode == o.tile_mode &&
            subtree_bytes == o.subtree_bytes && warp_teams == o.warp_teams &&
            sm_count == o.sm_count && graph_hi_occupancy == o.graph_hi_occupancy &&
-           plan_trees == o.plan_trees;
+           plan_trees == o.plan_trees && compact == o.compact;
   }
 };
 

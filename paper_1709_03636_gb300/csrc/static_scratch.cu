@@ -70,57 +70,70 @@ extern "C" qtc_status qtc_qaoa_expectation_static(qtc_batch* b, const double* pa
     std::lock_guard<std::mutex> lock(g_mutex);
     DeviceSetup& setup = setup_device(dev);
     const size_t max_dyn = max_dynamic_smem(setup.smem_optin);
-    const HostProgram& hp = host_program(b, dtype, want_grad, max_dyn);
-    if (hp.graph)
+    struct Layout {   // of one call inside the array
+      size_t tasks, ops, wsteps, coef, weights, results, acc, counters, total;
+    };
+    auto layout_of = [](const HostProgram& hp) {
+      const size_t P = hp.n_params, N = hp.n_nets;
+      Layout l;
+      l.tasks = align256(sizeof(GateEntryDev) * hp.gates.size());
+      l.ops = align256(l.tasks + sizeof(TaskDev) * hp.tasks.size());
+      l.wsteps = align256(l.ops + sizeof(uint4) * hp.stream.size());
+      l.coef = align256(l.wsteps + sizeof(WStep) * hp.wsteps.size());
+      l.weights = align256(l.coef + hp.coef.size());
+      l.results = align256(l.weights + sizeof(double) * N);
+      // the FP64 sums and the counters sit together: one clear per call
+      l.acc = align256(l.results + sizeof(double) * N * (2 + 2 * P));
+      l.counters = l.acc + ((sizeof(double) * (1 + P) + 15) & ~size_t(15));
+      l.total = l.counters + sizeof(unsigned int) * 4;
+      return l;
+    };
+    const HostProgram* prog = &host_program(b, dtype, want_grad, max_dyn);
+    if (prog->graph)
       fail(QTC_ERR_UNSUPPORTED,
            "this batch has networks larger than one CTA's shared memory; use "
            "qtc_qaoa_expectation_device with an arena");
-    const int P = hp.n_params, N = hp.n_nets, G = (int)hp.gates.size();
-
-    // layout of one call inside the array
-    const size_t o_gates = 0;
-    const size_t o_tasks = align256(o_gates + sizeof(GateEntryDev) * G);
-    const size_t o_ops = align256(o_tasks + sizeof(TaskDev) * hp.tasks.size());
-    const size_t o_wsteps = align256(o_ops + sizeof(uint4) * hp.stream.size());
-    const size_t o_coef = align256(o_wsteps + sizeof(WStep) * hp.wsteps.size());
-    const size_t o_weights = align256(o_coef + hp.coef.size());
-    const size_t o_results = align256(o_weights + sizeof(double) * N);
-    // the FP64 sums and the counters sit together: one clear per call
-    const size_t o_acc = align256(o_results + sizeof(double) * (size_t)N * (2 + 2 * P));
-    const size_t o_counters = o_acc + ((sizeof(double) * (1 + P) + 15) & ~size_t(15));
-    const size_t total = o_counters + sizeof(unsigned int) * 4;
-    if (total > kScratchBytes)
+    Layout lay = layout_of(*prog);
+    if (lay.total > kScratchBytes && !prog->warp_teams) {
+      ProgramOptions small;
+      small.compact = true;
+      prog = &host_program(b, dtype, want_grad, max_dyn, small);
+      lay = layout_of(*prog);
+    }
+    if (lay.total > kScratchBytes)
       fail(QTC_ERR_ARENA,
            "this batch needs %zu bytes of device scratch; the static scratch array holds %zu "
            "bytes (use qtc_qaoa_expectation_device with an arena instead)",
-           total, kScratchBytes);
+           lay.total, kScratchBytes);
+    const HostProgram& hp = *prog;
+    const int P = hp.n_params, N = hp.n_nets, G = (int)hp.gates.size();
 
     char* base = (char*)setup.scratch;
     cudaStream_t s = (cudaStream_t)stream;
     if (setup.resident != hp.serial) {
-      cuda_check(cudaMemcpyAsync(base + o_gates, hp.gates.data(), sizeof(GateEntryDev) * G,
+      cuda_check(cudaMemcpyAsync(base, hp.gates.data(), sizeof(GateEntryDev) * G,
                                  cudaMemcpyHostToDevice, s), "upload gates");
-      cuda_check(cudaMemcpyAsync(base + o_tasks, hp.tasks.data(),
+      cuda_check(cudaMemcpyAsync(base + lay.tasks, hp.tasks.data(),
                                  sizeof(TaskDev) * hp.tasks.size(), cudaMemcpyHostToDevice, s),
                  "upload tasks");
       if (!hp.stream.empty())
-        cuda_check(cudaMemcpyAsync(base + o_ops, hp.stream.data(),
+        cuda_check(cudaMemcpyAsync(base + lay.ops, hp.stream.data(),
                                    sizeof(uint4) * hp.stream.size(), cudaMemcpyHostToDevice, s),
                    "upload programs");
       if (!hp.wsteps.empty())
-        cuda_check(cudaMemcpyAsync(base + o_wsteps, hp.wsteps.data(),
+        cuda_check(cudaMemcpyAsync(base + lay.wsteps, hp.wsteps.data(),
                                    sizeof(WStep) * hp.wsteps.size(),
                                    cudaMemcpyHostToDevice, s), "upload warp ops");
       if (!hp.coef.empty())
-        cuda_check(cudaMemcpyAsync(base + o_coef, hp.coef.data(), hp.coef.size(),
+        cuda_check(cudaMemcpyAsync(base + lay.coef, hp.coef.data(), hp.coef.size(),
                                    cudaMemcpyHostToDevice, s), "upload gate coefficients");
-      cuda_check(cudaMemcpyAsync(base + o_weights, hp.weights.data(), sizeof(double) * N,
+      cuda_check(cudaMemcpyAsync(base + lay.weights, hp.weights.data(), sizeof(double) * N,
                                  cudaMemcpyHostToDevice, s), "upload weights");
       setup.resident = hp.serial;
     }
     // the sums, the queue and the team counter must start at zero; the array
     // keeps whatever the previous call left there
-    cuda_check(cudaMemsetAsync(base + o_acc, 0, o_counters - o_acc + sizeof(unsigned int) * 4, s),
+    cuda_check(cudaMemsetAsync(base + lay.acc, 0, lay.counters - lay.acc + sizeof(unsigned int) * 4, s),
                "clear counters");
 
     int per_sm = 0;
@@ -129,7 +142,7 @@ extern "C" qtc_status qtc_qaoa_expectation_static(qtc_batch* b, const double* pa
                                    hp.block, &per_sm), "configure executor");
     if (per_sm < 1) fail(QTC_ERR_UNSUPPORTED, "executor does not fit on an SM");
     ProgramDev d{};
-    d.gates = (const GateEntryDev*)(base + o_gates);
+    d.gates = (const GateEntryDev*)(base);
     d.n_gates = G;
     for (int g = 0; g < G && g < kInlineGates; ++g) d.gates_inline[g] = hp.gates[g];
     d.table_elems = hp.table_elems;
@@ -139,19 +152,19 @@ extern "C" qtc_status qtc_qaoa_expectation_static(qtc_batch* b, const double* pa
     d.half_units = hp.half_units;
     d.lane_dots = hp.lane_dots;
     d.task_stride = hp.task_stride;
-    d.coef = base + o_coef;
-    d.tasks = (const TaskDev*)(base + o_tasks);
+    d.coef = base + lay.coef;
+    d.tasks = (const TaskDev*)(base + lay.tasks);
     d.n_tasks = (int)hp.tasks.size();
-    d.stream = (const uint4*)(base + o_ops);
-    d.wsteps = (const WStep*)(base + o_wsteps);
+    d.stream = (const uint4*)(base + lay.ops);
+    d.wsteps = (const WStep*)(base + lay.wsteps);
     d.n_params = P;
     d.n_nets = N;
-    d.weights = (const double*)(base + o_weights);
+    d.weights = (const double*)(base + lay.weights);
     d.params = params_dev;
-    d.results = (double*)(base + o_results);
-    d.acc = (double*)(base + o_acc);
+    d.results = (double*)(base + lay.results);
+    d.acc = (double*)(base + lay.acc);
     d.out = out_dev;
-    d.counters = (unsigned int*)(base + o_counters);
+    d.counters = (unsigned int*)(base + lay.counters);
     d.want_grad = hp.want_grad;
     d.qaoa_reduce = hp.qaoa_reduce;
     const int ctas = ((int)hp.tasks.size() + hp.n_teams - 1) / hp.n_teams;
