@@ -180,10 +180,8 @@ WaveHost assemble_wave(const std::vector<int>& nets, const std::vector<NetGraph>
   }
   auto lower = [&](int a, int b) { return rank[a] < rank[b] || (rank[a] == rank[b] && a > b); };
   std::priority_queue<int, std::vector<int>, decltype(lower)> ready(lower);
-  using Event = std::pair<double, int>;
+  using Event = std::tuple<double, int, uint32_t>;   // end time, unit, its tasks ending then
   std::priority_queue<Event, std::vector<Event>, std::greater<Event>> done;
-  std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
-  for (int i = 0; i < std::max(teams, 1); ++i) free_at.push(0.0);
   std::vector<uint32_t> next(U, 0), left(n_tasks);
   size_t total = 0;
   for (size_t i = 0; i < U; ++i) {
@@ -191,28 +189,36 @@ WaveHost assemble_wave(const std::vector<int>& nets, const std::vector<NetGraph>
     if (n_deps[i] == 0) ready.push((int)i);
   }
   w.tasks.reserve(total);
-  while (w.tasks.size() < total) {
-    const double now = free_at.top();
-    free_at.pop();
-    while (!done.empty() && done.top().first <= now) {
-      const int gid = done.top().second;
+  // (teams are counted and tasks that start together end as one event: walking the idle
+  // teams at every event, the lowering of a lone p=3 network, 5743 tasks on 608 teams,
+  // took 4.0 ms instead of 2.3)
+  uint32_t idle = (uint32_t)std::max(teams, 1);
+  for (double now = 0.0;;) {
+    while (idle > 0 && !ready.empty()) {
+      const int gid = ready.top();
+      const uint32_t n = std::min(idle, n_tasks[gid] - next[gid]);
+      GTask t = tmpl[gid];
+      for (uint32_t i = 0; i < n; ++i) {
+        if (t.kind != GT_SMEM) t.b = next[gid] + i;
+        w.tasks.push_back(t);
+      }
+      next[gid] += n;
+      if (next[gid] == n_tasks[gid]) ready.pop();
+      done.push({now + dur[gid], gid, n});
+      idle -= n;
+    }
+    if (w.tasks.size() == total) break;
+    if (done.empty()) fail(QTC_ERR_INVALID, "internal: units with unmet dependencies");
+    // to the next time at which tasks end: their teams are free, their units may be done
+    for (now = std::get<0>(done.top()); !done.empty() && std::get<0>(done.top()) <= now;) {
+      const int gid = std::get<1>(done.top());
+      const uint32_t n = std::get<2>(done.top());
       done.pop();
-      if (--left[gid] == 0)
+      idle += n;
+      if ((left[gid] -= n) == 0)
         for (int s : succ[gid])
           if (--n_deps[s] == 0) ready.push(s);
     }
-    if (ready.empty()) {
-      if (done.empty()) fail(QTC_ERR_INVALID, "internal: units with unmet dependencies");
-      free_at.push(done.top().first);   // idle until the next task ends
-      continue;
-    }
-    const int gid = ready.top();
-    GTask t = tmpl[gid];
-    if (t.kind != GT_SMEM) t.b = next[gid];
-    w.tasks.push_back(t);
-    if (++next[gid] == n_tasks[gid]) ready.pop();
-    done.push({now + dur[gid], gid});
-    free_at.push(now + dur[gid]);
   }
   return w;
 }
