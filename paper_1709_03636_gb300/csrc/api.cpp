@@ -870,19 +870,21 @@ const HostProgram& qtc::host_program(qtc_batch* b, int dtype, int want_grad,
   for (int i = 0; i < N; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(),
                    [&](int x, int y) { return b->plans[x].cmacs > b->plans[y].cmacs; });
-  bool all_fit = !opts.force_graph;
-  for (int i : order) {
-    if (!all_fit) break;
-    LoweredNet ln = lower_smem(b->plans[i], leaf_gate[i], val_off, der_off, table_elems,
-                               want_grad != 0, max_elems);
-    if (!ln.fits) {
-      all_fit = false;
-      break;
-    }
+  // (networks on several threads: the 250 of p=2 n=100 take 0.1 s in all, 0.48 on one)
+  std::atomic<bool> all_fit{!opts.force_graph};
+  std::vector<LoweredNet> lowered(N);
+  parallel_for(N, [&](int k) {
+    if (!all_fit) return;   // (largest first: a network that does not fit is found at once)
+    lowered[k] = lower_smem(b->plans[order[k]], leaf_gate[order[k]], val_off, der_off, table_elems,
+                            want_grad != 0, max_elems);
+    if (!lowered[k].fits) all_fit = false;
+  });
+  for (int k = 0; all_fit && k < N; ++k) {
+    const LoweredNet& ln = lowered[k];
     TaskDev t{};
     t.op_begin = (uint32_t)hp->ops.size();
     t.op_count = (uint32_t)ln.ops.size();
-    t.net = (uint32_t)i;
+    t.net = (uint32_t)order[k];
     t.arena_elems = ln.arena_elems;
     hp->tasks.push_back(t);
     hp->ops.insert(hp->ops.end(), ln.ops.begin(), ln.ops.end());
@@ -958,28 +960,35 @@ const HostProgram& qtc::host_program(qtc_batch* b, int dtype, int want_grad,
     const uint32_t private_below = pass == 0 ? UINT32_MAX : 32u;
     WarpCand c;
     c.tasks = hp->tasks;
-    bool fit = true;
-    for (TaskDev& t : c.tasks) {
+    std::vector<std::vector<WStep>> steps(c.tasks.size());
+    std::atomic<bool> fit{true};
+    parallel_for((int)c.tasks.size(), [&](int i) {
+      TaskDev& t = c.tasks[i];
+      if (!fit) return;
       std::vector<SOp> net_ops(hp->ops.begin() + t.op_begin,
                                hp->ops.begin() + t.op_begin + t.op_count);
-      const uint32_t begin = (uint32_t)c.wsteps.size();
       if (!reuse) {
         LoweredNet ln = lower_smem(b->plans[t.net], leaf_gate[t.net], val_off, der_off,
                                    table_elems, want_grad != 0, max_elems, private_below);
         if (!ln.fits || (size_t)table_elems + ln.arena_elems > 0xffffu) {
           fit = false;
-          break;
+          return;
         }
         t.arena_elems = ln.arena_elems;
         net_ops = std::move(ln.ops);
       }
-      build_warp_steps(net_ops, table_elems, t.arena_elems, c.wsteps);
+      build_warp_steps(net_ops, table_elems, t.arena_elems, steps[i]);
+    });
+    if (!fit) continue;
+    for (size_t i = 0; i < c.tasks.size(); ++i) {
+      TaskDev& t = c.tasks[i];
       c.max_arena = std::max(c.max_arena, t.arena_elems);
-      t.op_begin = begin;
-      t.op_count = (uint32_t)c.wsteps.size() - begin;
+      t.op_begin = (uint32_t)c.wsteps.size();
+      t.op_count = (uint32_t)steps[i].size();
       c.max_steps = std::max(c.max_steps, t.op_count);
+      c.wsteps.insert(c.wsteps.end(), steps[i].begin(), steps[i].end());
     }
-    if (fit) cands.push_back(std::move(c));
+    cands.push_back(std::move(c));
   }
   // (complex128 programs that need streamed steps or fewer teams per CTA
   // measured slower on warps than on a CTA per network: they stay staged
@@ -1074,33 +1083,39 @@ const HostProgram& qtc::host_program(qtc_batch* b, int dtype, int want_grad,
     fail(QTC_ERR_UNSUPPORTED, "program needs %zu bytes of shared memory (limit %zu)", hp->smem,
          max_dynamic);
   if (!hp->warp_teams) {
-    std::vector<std::vector<SOp>> progs;
-    size_t raw = 0;
-    for (const TaskDev& t : hp->tasks) {
-      progs.emplace_back(hp->ops.begin() + t.op_begin, hp->ops.begin() + t.op_begin + t.op_count);
-      raw += t.op_count * sizeof(SOp);
-      schedule_cta_ops(progs.back(), table_elems, kExecBlock / 32);
-      validate_cta_ops(progs.back().data(), progs.back().size(), table_elems, t.arena_elems, 0, P,
+    const int n_progs = (int)hp->tasks.size();
+    std::vector<std::vector<SOp>> progs(n_progs);
+    std::vector<std::vector<uint4>> streams(n_progs);
+    auto write_stream = [&](int i, bool smallest) {
+      TaskDev& t = hp->tasks[i];
+      std::vector<uint4>& s = streams[i];
+      s.clear();
+      t.op_count = smallest
+                       ? build_smallest_stream(progs[i], hp->half_units, hp->lane_dots, s)
+                       : build_cta_stream(progs[i], hp->half_units, kLaneLimit, hp->lane_dots, s);
+      validate_cta_stream(s.data(), s.size(), t.op_count, hp->half_units, table_elems,
+                          t.arena_elems, P);
+    };
+    const size_t raw = hp->ops.size() * sizeof(SOp);
+    parallel_for(n_progs, [&](int i) {
+      const TaskDev& t = hp->tasks[i];
+      progs[i].assign(hp->ops.begin() + t.op_begin, hp->ops.begin() + t.op_begin + t.op_count);
+      schedule_cta_ops(progs[i], table_elems, kExecBlock / 32);
+      validate_cta_ops(progs[i].data(), progs[i].size(), table_elems, t.arena_elems, 0, P,
                        kExecBlock / 32);
-    }
-    hp->ops.clear();
-    for (const auto& p : progs) hp->ops.insert(hp->ops.end(), p.begin(), p.end());
+      write_stream(i, opts.compact);
+    });
+    size_t units = 0;
+    for (const auto& s : streams) units += s.size();
     // lanes take more memory than records for the wider ops: not where that makes a large
     // program larger than its ops
-    for (const bool smallest : {false, true}) {
-      if (opts.compact && !smallest) continue;
-      hp->stream.clear();
-      for (size_t i = 0; i < progs.size(); ++i) {
-        TaskDev& t = hp->tasks[i];
-        t.op_begin = (uint32_t)hp->stream.size();
-        t.op_count = smallest ? build_smallest_stream(progs[i], hp->half_units, hp->lane_dots,
-                                                      hp->stream)
-                              : build_cta_stream(progs[i], hp->half_units, kLaneLimit,
-                                                 hp->lane_dots, hp->stream);
-        validate_cta_stream(hp->stream.data() + t.op_begin, hp->stream.size() - t.op_begin,
-                            t.op_count, hp->half_units, table_elems, t.arena_elems, P);
-      }
-      if (hp->stream.size() * sizeof(uint4) <= std::max<size_t>(raw, 1u << 20)) break;
+    if (!opts.compact && units * sizeof(uint4) > std::max<size_t>(raw, 1u << 20))
+      parallel_for(n_progs, [&](int i) { write_stream(i, true); });
+    hp->ops.clear();
+    for (int i = 0; i < n_progs; ++i) {
+      hp->tasks[i].op_begin = (uint32_t)hp->stream.size();
+      hp->ops.insert(hp->ops.end(), progs[i].begin(), progs[i].end());
+      hp->stream.insert(hp->stream.end(), streams[i].begin(), streams[i].end());
     }
   }
   b->host_programs.push_back(std::move(hp));

@@ -1,10 +1,7 @@
 // Host side of the graph executor: per-network units -> waves of tasks.
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <queue>
-#include <system_error>
-#include <thread>
 #include <tuple>
 
 #include "qtc_internal.h"
@@ -507,7 +504,6 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
   if (lim.min_chunks < 16 || opts.compact) lim.min_chunks = 1;
   lim.stage_rows = !opts.compact;
   std::vector<NetGraph> graphs(N);
-  std::vector<Error> errors(N, Error{QTC_OK, ""});
   auto lower_one = [&](int i) {
     // a network that fits whole in shared memory stays one fused task
     LoweredNet ln = lower_smem(plans[i], leaf_gate[i], val_off, der_off, hp.table_elems,
@@ -536,30 +532,7 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
     check_global_placement(g);
     graphs[i] = std::move(g);
   };
-  {
-    const unsigned hw = std::max(1u, std::min({32u, std::thread::hardware_concurrency(),
-                                               (unsigned)N}));
-    std::atomic<int> next{0};
-    auto work = [&] {
-      for (int i = next++; i < N; i = next++) try {
-          lower_one(i);
-        } catch (const Error& e) {
-          errors[i] = e;
-        } catch (const std::exception& e) {
-          errors[i] = Error{QTC_ERR_INVALID, e.what()};
-        }
-    };
-    std::vector<std::thread> pool;
-    try {
-      for (unsigned t = 1; t < hw; ++t) pool.emplace_back(work);
-    } catch (const std::system_error&) {
-      // fewer threads than asked for: the ones there are do the work
-    }
-    work();
-    for (auto& th : pool) th.join();
-  }
-  for (const Error& e : errors)
-    if (e.status != QTC_OK) throw e;
+  parallel_for(N, lower_one);
   for (const NetGraph& g : graphs) {
     hp.max_checkpoint_segments = std::max(hp.max_checkpoint_segments, g.checkpoint_segments);
     hp.sum_global_elems += g.global_elems;

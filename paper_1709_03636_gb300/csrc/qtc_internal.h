@@ -1,9 +1,13 @@
 // Internal host-side structures of the contraction engine.
 #pragma once
 
+#include <algorithm>
+#include <atomic>
 #include <complex>
 #include <cstdint>
+#include <exception>
 #include <string>
+#include <thread>
 #include <utility>
 #include <vector>
 
@@ -52,6 +56,33 @@ qtc_status guarded(F&& f) {
     set_last_error(e.what());
     return QTC_ERR_INVALID;
   }
+}
+
+// Runs f(0) .. f(n - 1) on several host threads (fewer where the system refuses more).
+// Every call has ended on return; the exception of the lowest index is thrown again.
+template <typename F>
+void parallel_for(int n, F&& f) {
+  std::vector<std::exception_ptr> errors(n);
+  std::atomic<int> next{0};
+  auto work = [&]() noexcept {
+    for (int i = next++; i < n; i = next++) try {
+        f(i);
+      } catch (...) {
+        errors[i] = std::current_exception();
+      }
+  };
+  const unsigned want = std::min({32u, std::thread::hardware_concurrency(), (unsigned)n});
+  std::vector<std::thread> pool;
+  try {
+    pool.reserve(want);
+    for (unsigned t = 1; t < want; ++t) pool.emplace_back(work);
+  } catch (const std::exception&) {
+    // the threads there are do the work
+  }
+  work();
+  for (std::thread& th : pool) th.join();
+  for (const std::exception_ptr& e : errors)
+    if (e) std::rethrow_exception(e);
 }
 
 // Restores the caller's current device on scope exit.
