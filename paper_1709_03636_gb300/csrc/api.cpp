@@ -586,7 +586,7 @@ extern "C" qtc_status qtc_plan_execution_tree(const qtc_plan* p, int dtype, qtc_
     if (dtype != QTC_C128 && dtype != QTC_C64 && dtype != QTC_SPLIT_BF16)
       fail(QTC_ERR_INVALID, "unknown dtype %d", dtype);
     auto q = std::make_unique<qtc_plan>();
-    q->plan = execution_plan(p->plan, tree_model(dtype));
+    q->plan = execution_plan(p->plan, dtype, true);
     *out = q.release();
   });
 }
@@ -806,7 +806,7 @@ extern "C" qtc_status qtc_batch_execution_trees(const qtc_batch* b, int dtype, q
     s->qaoa_reduce = b->qaoa_reduce;
     s->obs_edges = b->obs_edges;
     s->weights = b->weights;
-    for (const Plan& p : b->plans) s->plans.push_back(execution_plan(p, tree_model(dtype)));
+    for (const Plan& p : b->plans) s->plans.push_back(execution_plan(p, dtype, b->plans.size() == 1));
     *out = s.release();
   });
 }

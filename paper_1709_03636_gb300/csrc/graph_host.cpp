@@ -493,7 +493,6 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
     }
     return best;
   };
-  const TreeModel model = tree_model(hp.dtype);
   // A network's steps are cut finer, towards two tasks per SM, when few networks
   // share the device: one p=3 edge network 551 -> 376 us (four tasks per SM 411, one
   // 370, a half 398; over nine edge networks of 32 to 60 vertices two is the best or
@@ -519,7 +518,7 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
     }
     NetGraph g;
     g.fits = false;
-    if (!opts.plan_trees && !opts.compact) g = lower_network(i, execution_plan(plans[i], model));
+    if (!opts.plan_trees && !opts.compact) g = lower_network(i, execution_plan(plans[i], hp.dtype, N == 1));
     if (!g.fits || over(g)) {
       // the plan's own tree, where the rearranged one cannot be lowered or
       // needs more memory than a wave may take

@@ -288,8 +288,6 @@ std::vector<Step> eliminate(const Network& net, const std::vector<int>& order) {
   return st.steps;
 }
 
-}  // namespace
-
 // Per-step label layout.  A label's death is the step that sums it; every
 // intermediate stores its labels by decreasing death step (the label that
 // survives longest is bit 0), so operands of later steps share low bits.
@@ -325,6 +323,8 @@ void layout_labels(Plan& plan) {
   plan.cmacs = c.flops;
   plan.bytes_c64 = 8.0 * c.elems;
 }
+
+}  // namespace
 
 Plan make_plan(const Network& net, const qtc_plan_opts& o) {
   if (net.leaves.empty()) fail(QTC_ERR_INVALID, "empty network");

@@ -6,6 +6,8 @@
 #include <complex>
 #include <cstdint>
 #include <exception>
+#include <memory>
+#include <mutex>
 #include <string>
 #include <thread>
 #include <utility>
@@ -157,6 +159,17 @@ struct Step {
   int a, b;        // operand tensor ids
 };
 
+// The tree of execution_plan, searched for once for all plans of one structure (copies
+// of a plan, and plans of other values that reuse its tree).
+struct ExecutionTree {
+  std::mutex mutex;
+  bool known = false;
+  std::vector<Step> steps;   // empty: the plan's own
+  std::vector<std::vector<int>> labels;
+  int max_rank = 0;
+  double cmacs = 0, bytes_c64 = 0;
+};
+
 struct Plan {
   Network net;
   std::vector<Step> steps;
@@ -165,24 +178,15 @@ struct Plan {
   std::vector<std::vector<int>> labels;
   int max_rank = 0;
   double cmacs = 0, bytes_c64 = 0, lg_width = 0;
+  std::shared_ptr<ExecutionTree> tree = std::make_shared<ExecutionTree>();
 };
 
 Plan make_plan(const Network& net, const qtc_plan_opts& opts);
-// Storage order of every tensor's labels and the plan's costs, from its steps.
-void layout_labels(Plan& plan);
 
-// What a step costs on the device, for choosing the tree to execute.
-struct TreeModel {
-  double elem = 8;             // bytes per element
-  double bytes_per_ns = 6000;  // memory, all SMs
-  double macs_per_ns = 3000;   // complex multiply-adds, all SMs
-  double step_ns = 1;          // per step, over the networks that run beside it
-  int small_rank = 10;         // trees of tensors up to this rank stay as they are
-};
-// The model of an element type (qtc_dtype).
-TreeModel tree_model(int dtype);
-// The plan with a tree rearranged for execution (same network, same scalar).
-Plan execution_plan(const Plan& plan, const TreeModel& model);
+// The plan with a tree rearranged for execution in an element type (same network, same
+// scalar; single precision keeps the plan's own).  alone: the caller has no other
+// networks to work on, so the search may take another thread.
+Plan execution_plan(const Plan& plan, int dtype, bool alone);
 
 // ---- leaf tensors as coefficients (gate_coef.cpp) ---------------------------
 // A, B, C (2^rank each) with element = A cos(t/2) + B sin(t/2) + C.

@@ -25,6 +25,11 @@ constexpr int kMaxFrontier = 8;   // subtrees rearranged at once: up to 3^8 spli
 // different local optima, the better one is taken.
 constexpr int kSchedule[2][6] = {{8, 8, 8, 8, 8, 8}, {4, 5, 6, 7, 8, 8}};
 constexpr double kWorthIt = 0.03; // share of the tree's time below which steps are left alone
+constexpr int kSmallRank = 10;    // trees of tensors up to this rank stay as they are
+// What a step costs on the device (complex128): bytes moved by all SMs per ns,
+// multiply-adds per ns on the narrow FP64 pipe (160 at its peak; fewer of them is what
+// pays), and ns per step over the networks that run beside it.
+constexpr double kElemBytes = 16, kBytesPerNs = 6000, kMacsPerNs = 150, kStepNs = 1;
 
 struct Tree {
   int n_leaves = 0, root = 0, words = 0;
@@ -47,18 +52,18 @@ constexpr int kMaxStepLabels = 64;
 // Expected time (ns over the whole device) of one step, from tables over the
 // ranks of its tensors and the number of its labels.
 struct StepTimes {
-  double move[kMaxStepLabels + 1], work[kMaxStepLabels + 1], fixed;
-  explicit StepTimes(const TreeModel& m) : fixed(m.step_ns) {
+  double move[kMaxStepLabels + 1], work[kMaxStepLabels + 1];
+  StepTimes() {
     for (int i = 0; i <= kMaxStepLabels; ++i) {
-      move[i] = m.elem * std::ldexp(1.0, i) / m.bytes_per_ns;
-      work[i] = std::ldexp(1.0, i) / m.macs_per_ns;
+      move[i] = kElemBytes * std::ldexp(1.0, i) / kBytesPerNs;
+      work[i] = std::ldexp(1.0, i) / kMacsPerNs;
     }
   }
   double operator()(int ra, int rb, int rc, int all) const {
     // the larger of moving and computing, and part of the other (they overlap
     // within a step, but not perfectly)
     const double mv = move[ra] + move[rb] + move[rc], wk = work[all];
-    return std::max(mv, wk) + 0.25 * std::min(mv, wk) + fixed;
+    return std::max(mv, wk) + 0.25 * std::min(mv, wk) + kStepNs;
   }
 };
 
@@ -142,18 +147,30 @@ bool rearrange(Tree& t, int node, int width, const StepTimes& time, double least
   }
   if (t.seen[node] == sign) return false;
   t.seen[node] = sign;
+  // made: a subset's cost and the move of its result, what any split above it pays
+  double made[1 << kMaxFrontier];
+  for (int i = 0; i < k; ++i) made[1 << i] = time.move[rank[1 << i]];
   for (int s = 3; s <= all; ++s) {
-    // (a subset whose result alone takes longer is no use either)
-    if (!(s & (s - 1)) || time.move[rank[s]] >= old) continue;
+    if (!(s & (s - 1))) continue;
+    made[s] = HUGE_VAL;
+    // (what the subset may cost to be of use to the whole)
+    const double out_move = time.move[rank[s]];
+    const double useful = s == all ? old : old - out_move - time.move[rank[all]];
+    if (out_move >= useful) continue;
+    double least_made = useful - out_move;
     for (int a = (s - 1) & s; a; a = (a - 1) & s) {
       const int b = s ^ a;
       if (a < b) break;            // the other half of the splits
-      const double parts = cost[a] + cost[b];
-      if (parts >= cost[s] || parts >= old) continue;   // `old`: no use to the whole
-      const double c =
-          parts + time(rank[a], rank[b], rank[s], __builtin_popcountll(open[a] | open[b]));
-      if (c < cost[s]) cost[s] = c, split[s] = a;
+      if (made[a] + made[b] >= least_made) continue;
+      const double c = cost[a] + cost[b] +
+                       time(rank[a], rank[b], rank[s], __builtin_popcountll(open[a] | open[b]));
+      if (c < cost[s]) {
+        cost[s] = c;
+        split[s] = a;
+        least_made = std::min(c, useful) - out_move;
+      }
     }
+    made[s] = cost[s] + out_move;
   }
   if (!(cost[all] < 0.999 * old)) return false;
   // rebuild with the same inner nodes, `node` staying the top
@@ -178,46 +195,30 @@ bool rearrange(Tree& t, int node, int width, const StepTimes& time, double least
 
 }  // namespace
 
-TreeModel tree_model(int dtype) {
-  TreeModel m;
-  m.elem = (double)elem_bytes(dtype);
-  if (dtype == QTC_C128) {
-    // multiply-adds run on the narrow FP64 pipe (0.16 per ps at its peak): fewer
-    // of them is what pays
-    m.macs_per_ns = 150;
-  } else {
-    // Single precision keeps the plan's own order of every sum: expectation
-    // values are often far below one (p=1 on a 7-regular graph: under 5e-3 for a
-    // third of all angles), and another tree moves them by their whole rounding
-    // error (1.5e-3 relative seen on 7-regular n=26), for all that it was 2.0x
-    // faster there and 1.7x on p=3 n=60.
-    m.small_rank = 1 << 20;
-  }
-  return m;
-}
+namespace {
 
-Plan execution_plan(const Plan& plan, const TreeModel& m) {
+// The best tree found for `plan`; no steps when that is its own.
+void search_tree(const Plan& plan, bool alone, ExecutionTree& out) {
   const int L = (int)plan.net.leaves.size(), S = (int)plan.steps.size();
-  if (plan.max_rank <= m.small_rank) return plan;
-  Tree t;
-  t.n_leaves = L;
-  t.root = L + S - 1;
-  t.words = (plan.net.n_labels + 63) / 64;
-  t.left.assign(L + S, -1);
-  t.right.assign(L + S, -1);
-  t.bits.assign((size_t)(L + S) * t.words, 0);
-  t.seen.assign(L + S, 0);
+  Tree given;
+  given.n_leaves = L;
+  given.root = L + S - 1;
+  given.words = (plan.net.n_labels + 63) / 64;
+  given.left.assign(L + S, -1);
+  given.right.assign(L + S, -1);
+  given.bits.assign((size_t)(L + S) * given.words, 0);
+  given.seen.assign(L + S, 0);
   for (int i = 0; i < L + S; ++i)
-    for (int x : plan.labels[i]) t.labels(i)[x >> 6] |= 1ull << (x & 63);
+    for (int x : plan.labels[i]) given.labels(i)[x >> 6] |= 1ull << (x & 63);
   for (int s = 0; s < S; ++s) {
-    t.left[L + s] = plan.steps[s].a;
-    t.right[L + s] = plan.steps[s].b;
+    given.left[L + s] = plan.steps[s].a;
+    given.right[L + s] = plan.steps[s].b;
   }
   for (int x = L; x < L + S; ++x)
-    if (labels_of_step(t, x) > kMaxStepLabels) return plan;
-  const StepTimes time(m);
-  std::vector<int> order;          // inner nodes, children before parents
-  auto walk = [&](Tree& t) {
+    if (labels_of_step(given, x) > kMaxStepLabels) return;
+  const StepTimes time;
+  // inner nodes, children before parents; the time of all steps
+  auto walk = [&](Tree& t, std::vector<int>& order) {
     order.clear();
     std::vector<int> todo{t.root};
     while (!todo.empty()) {        // parents first, then reversed
@@ -233,40 +234,92 @@ Plan execution_plan(const Plan& plan, const TreeModel& m) {
     for (int x : order) total += step_of(t, x, time);
     return total;
   };
-  const Tree given = t;
-  double best = walk(t);
-  bool changed = false;
-  for (const auto& schedule : kSchedule) {
-    Tree u = given;
-    for (int width : schedule) {
-      const double least = kWorthIt * walk(u);
+  Tree found[2];
+  std::vector<int> orders[2];
+  double totals[2];
+  auto search = [&](int k) {
+    Tree& u = found[k] = given;
+    std::vector<int>& order = orders[k];
+    for (int width : kSchedule[k]) {
+      const double least = kWorthIt * walk(u, order);
       bool moved = false;
       for (auto it = order.rbegin(); it != order.rend(); ++it) {
         const int x = *it;
-        if (std::max({u.rank(x), u.rank(u.left[x]), u.rank(u.right[x])}) < m.small_rank) continue;
+        if (std::max({u.rank(x), u.rank(u.left[x]), u.rank(u.right[x])}) < kSmallRank) continue;
         if (rearrange(u, x, width, time, least)) moved = true;
       }
       if (!moved && width == kMaxFrontier) break;
     }
-    const double total = walk(u);
-    if (total < best) {
-      best = total;
-      t = std::move(u);
-      changed = true;
-    }
+    totals[k] = walk(u, order);
+  };
+  if (alone) {
+    parallel_for(2, search);
+  } else {
+    search(0);
+    search(1);
   }
-  if (!changed) return plan;
-  walk(t);
+  const int best = totals[1] < totals[0] ? 1 : 0;
+  {
+    std::vector<int> order;
+    if (!(totals[best] < walk(given, order))) return;
+  }
+  // its steps, and the labels in storage order as layout_labels gives them (a label
+  // that survives longer comes first), from the label sets at hand
+  Tree& t = found[best];
+  const std::vector<int>& nodes = orders[best];
+  std::vector<int> id(L + S, -1), death(plan.net.n_labels, S);
+  out.labels.assign(plan.labels.begin(), plan.labels.begin() + L);
+  out.labels.resize(L + S);
+  for (int i = 0; i < L; ++i) id[i] = i;
+  auto each = [&](uint64_t bits, int w, auto&& f) {
+    for (; bits; bits &= bits - 1) f(64 * w + __builtin_ctzll(bits));
+  };
+  double elems = 0;
+  for (int s = 0; s < S; ++s) {
+    const int x = nodes[s], a = t.left[x], b = t.right[x];
+    id[x] = L + s;
+    out.steps.push_back({id[a], id[b]});
+    for (int w = 0; w < t.words; ++w)
+      each((t.labels(a)[w] | t.labels(b)[w]) & ~t.labels(x)[w], w, [&](int l) { death[l] = s; });
+    out.cmacs += std::ldexp(1.0, labels_of_step(t, x));
+    elems += std::ldexp(1.0, t.rank(a)) + std::ldexp(1.0, t.rank(b)) + std::ldexp(1.0, t.rank(x));
+    out.max_rank = std::max(out.max_rank, t.rank(x));
+  }
+  out.bytes_c64 = 8.0 * elems;
+  for (int s = 0; s < S; ++s) {
+    std::vector<int>& r = out.labels[L + s];
+    for (int w = 0; w < t.words; ++w)
+      each(t.labels(nodes[s])[w], w, [&](int l) { r.push_back(l); });
+    std::sort(r.begin(), r.end(), [&](int x, int y) {
+      if (death[x] != death[y]) return death[x] > death[y];
+      return x < y;
+    });
+  }
+}
+
+}  // namespace
+
+Plan execution_plan(const Plan& plan, int dtype, bool alone) {
+  // Single precision keeps the plan's own order of every sum: expectation values are
+  // often far below one (p=1 on a 7-regular graph: under 5e-3 for a third of all
+  // angles), and another tree moves them by their whole rounding error (1.5e-3 relative
+  // seen on 7-regular n=26), for all that it was 2.0x faster there and 1.7x on p=3 n=60.
+  if (dtype != QTC_C128 || plan.max_rank <= kSmallRank) return plan;
+  ExecutionTree& tree = *plan.tree;
+  std::lock_guard<std::mutex> lock(tree.mutex);
+  if (!tree.known) {
+    search_tree(plan, alone, tree);
+    tree.known = true;
+  }
+  if (tree.steps.empty()) return plan;
   Plan out;
   out.net = plan.net;
   out.lg_width = plan.lg_width;
-  std::vector<int> id(L + S, -1);
-  for (int i = 0; i < L; ++i) id[i] = i;
-  for (int x : order) {
-    id[x] = L + (int)out.steps.size();
-    out.steps.push_back({id[t.left[x]], id[t.right[x]]});
-  }
-  layout_labels(out);
+  out.steps = tree.steps;
+  out.labels = tree.labels;
+  out.max_rank = tree.max_rank;
+  out.cmacs = tree.cmacs;
+  out.bytes_c64 = tree.bytes_c64;
   return out;
 }
 
