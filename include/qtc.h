@@ -316,8 +316,7 @@ qtc_status qtc_batch_partition(const qtc_batch* b, int n_parts, int want_grad,
 qtc_status qtc_batch_subset(const qtc_batch* b, const int32_t* nets, int k, qtc_batch** out);
 
 /* Builds, validates and describes the batch's device program on the host
- * only (no GPU call), along the plans' own contraction trees (an engine's graph
- * executor runs those of qtc_batch_execution_trees): every access range, counter and dependency order of a
+ * only (no GPU call): every access range, counter and dependency order of a
  * graph program is checked against its buffers.  force_graph, small_rank and
  * max_wave_bytes as in qtc_engine_set_graph_options / qtc_engine_set_limits;
  * smem_limit: shared memory per CTA to plan for (0: 227 KiB). */

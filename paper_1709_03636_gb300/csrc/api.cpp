@@ -203,7 +203,6 @@ extern "C" qtc_status qtc_engine_create(int device, void* arena, size_t arena_by
     cuda_check(cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device), "SM count");
     e->sm_count = v;
     e->options.sm_count = v;
-    e->options.plan_trees = false;
     cuda_check(cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, device),
                "shared memory limit");
     e->smem_optin = (size_t)v;

@@ -518,7 +518,7 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
     }
     NetGraph g;
     g.fits = false;
-    if (!opts.plan_trees && !opts.compact) g = lower_network(i, execution_plan(plans[i], hp.dtype, N == 1));
+    if (!opts.compact) g = lower_network(i, execution_plan(plans[i], hp.dtype, N == 1));
     if (!g.fits || over(g)) {
       // the plan's own tree, where the rearranged one cannot be lowered or
       // needs more memory than a wave may take

@@ -354,9 +354,7 @@ struct ProgramOptions {
                                    // 2: per warp, steps always streamed
   int sm_count = 152;              // SMs of the device the program is laid out for
   bool graph_hi_occupancy = false; // graph executor: the five-CTAs-per-SM instantiation
-  bool plan_trees = true;          // graph executor: contract the plans' own trees; false
-                                   // (what engines run): execution_plan's
-  bool compact = false;            // the smallest program tables (implies plan_trees): few lanes
+  bool compact = false;            // the smallest program tables: the plans' own trees, few lanes
                                    // in the streams, no steps cut finer for few networks
   bool operator==(const ProgramOptions& o) const {
     return wave_cap_bytes == o.wave_cap_bytes && force_graph == o.force_graph &&
@@ -364,7 +362,7 @@ struct ProgramOptions {
            tile_mode == o.tile_mode &&
            subtree_bytes == o.subtree_bytes && warp_teams == o.warp_teams &&
            sm_count == o.sm_count && graph_hi_occupancy == o.graph_hi_occupancy &&
-           plan_trees == o.plan_trees && compact == o.compact;
+           compact == o.compact;
   }
 };
 
