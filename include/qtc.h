@@ -425,6 +425,11 @@ qtc_status qtc_engine_set_tile_mode(qtc_engine* e, int mode);
 qtc_status qtc_selftest_tile_steps(qtc_batch* b, int dtype, int want_grad, int force_graph,
                                    int small_rank, int tile_mode, int max_bits,
                                    double* max_err, int32_t* n_checked);
+/* Host only: the staged long sums of the batch's graph program, as above.  counts: 4
+ * ints: steps that add sequentially, in eight accumulators, in four of pairs; of all of
+ * them those of more than 4096 values. */
+qtc_status qtc_selftest_stage_steps(qtc_batch* b, int dtype, int want_grad, int force_graph,
+                                    int small_rank, int32_t* counts);
 /* Host only: the order in which a team of the graph executor runs the batches of
  * a staged long sum, on a model in which threads meet at the barriers alone.
  * n_faults: accesses that another thread's may overtake (0 when sound). */

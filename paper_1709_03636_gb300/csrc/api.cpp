@@ -312,6 +312,25 @@ extern "C" qtc_status qtc_selftest_tile_steps(qtc_batch* b, int dtype, int want_
   });
 }
 
+extern "C" qtc_status qtc_selftest_stage_steps(qtc_batch* b, int dtype, int want_grad,
+                                               int force_graph, int small_rank,
+                                               int32_t* counts) {
+  return guarded([&] {
+    if (!b || !counts) fail(QTC_ERR_INVALID, "null argument");
+    ProgramOptions opts;
+    opts.force_graph = force_graph != 0;
+    opts.small_rank = small_rank;
+    const HostProgram& hp = host_program(b, dtype, want_grad, max_dynamic_smem(232448), opts);
+    std::fill(counts, counts + 4, 0);
+    for (const WaveHost& w : hp.waves)
+      for (const GStep& st : w.steps) {
+        if (!(st.flags & GSF_STAGE)) continue;
+        ++counts[st.flags & GSF_SUM8 ? 1 : st.flags & GSF_SUM_PAIR4 ? 2 : 0];
+        if ((1ull << st.ry) > kYTab) ++counts[3];
+      }
+  });
+}
+
 extern "C" qtc_status qtc_selftest_stage_schedule(int n_batches, int fold_every,
                                                   int32_t* n_faults) {
   return guarded([&] {
