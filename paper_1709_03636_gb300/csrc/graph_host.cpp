@@ -454,6 +454,14 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
   auto over = [&](const NetGraph& g) {
     return ((g.global_elems + 63) & ~uint64_t(63)) > cap_elems;
   };
+  // subtree arenas beyond the CTA's shared memory (beside the gate table and the least
+  // stage)
+  auto wide = [&](const NetGraph& g) {
+    for (const GUnit& u : g.units)
+      if ((size_t)hp.table_elems * elem + 2560 + 32 + (size_t)u.arena_elems * elem > max_dynamic)
+        return true;
+    return false;
+  };
   // one network's units, contracting `plan`'s tree
   auto lower_network = [&](int i, const Plan& plan) {
     // a subtree that does not fit its arena is cut into smaller ones
@@ -516,14 +524,14 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
       graphs[i].units.push_back(std::move(u));
       return;
     }
-    NetGraph g;
-    g.fits = false;
-    if (!opts.compact) g = lower_network(i, execution_plan(plans[i], hp.dtype, N == 1));
-    if (!g.fits || over(g)) {
+    const bool rearranged = hp.dtype == QTC_C128 && !opts.compact;
+    NetGraph g = rearranged ? lower_network(i, execution_plan(plans[i], hp.dtype, N == 1))
+                            : lower_network(i, plans[i]);
+    if (rearranged && (!g.fits || over(g) || wide(g))) {
       // the plan's own tree, where the rearranged one cannot be lowered or
-      // needs more memory than a wave may take
+      // needs more memory than a wave or a CTA may take
       NetGraph own = lower_network(i, plans[i]);
-      if (!g.fits || (own.fits && !over(own))) g = std::move(own);
+      if (!g.fits || (own.fits && !over(own) && !wide(own))) g = std::move(own);
     }
     if (!g.fits)
       fail(QTC_ERR_UNSUPPORTED, "network %d (max rank %d): %s", i, plans[i].max_rank,

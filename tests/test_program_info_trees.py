@@ -21,3 +21,16 @@ def test_complex128_programs_run_the_execution_trees(grad):
     own = batch.stats()["cmacs"]
     assert batch.execution_trees("c64").stats()["cmacs"] == own
     assert batch.execution_trees("c128").stats()["cmacs"] < 0.9 * own
+
+
+def test_a_tight_shared_memory_limit_takes_the_plans_own_tree():
+    """A rearranged tree may need a larger subtree arena than the plan's own: where a CTA
+    has no room for it, the network keeps the plan's, as single precision does anywhere."""
+    n = 16
+    edges = random_regular_graph(n, 3, n)
+    batch = q.Batch(q.Circuit.qaoa(n, edges, 1), edges[:4], lightcone=False, ordering="stoch")
+    free = batch.program_info("c128", True, force_graph=True)["smem_bytes"]
+    for limit in (free, 44000, 40000):
+        info = batch.program_info("c128", True, force_graph=True, smem_limit=limit + 16384)
+        assert info["graph"] and info["smem_bytes"] <= limit
+    assert free > 44000
