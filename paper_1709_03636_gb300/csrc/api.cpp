@@ -1048,9 +1048,9 @@ const HostProgram& qtc::host_program(qtc_batch* b, int dtype, int want_grad,
   }
   // A batch that leaves SMs idle takes fewer warps per CTA, as long as every CTA
   // has an SM of its own: the warps of a CTA share their SM's shared-memory and
-  // FP64 pipes.  Value + gradient, one warp against four: complex128 n=12 (18
-  // networks) 26.6 / 28.7 us, noisy n=51 (102 networks) 10.3 / 11.1 us, n=50 (75
-  // networks) 10.3 / 10.3 us.
+  // FP64 pipes.  The launch alone, value + gradient, one warp against four: complex128
+  // n=12 (18 networks) 26.6 / 28.7 us, noisy n=51 (102 networks) 10.3 / 11.1 us, n=50 (75
+  // networks) 10.3 / 10.3 us.  (Calls from the host take 33 to 48 us and do not show it.)
   for (const uint32_t stage = hp->stage_ops; ok && hp->n_teams > 1 &&
        2 * hp->tasks.size() <= (size_t)opts.sm_count * hp->n_teams;)
     ok = layout(true, stage, hp->n_teams / 2);
