@@ -539,7 +539,7 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
     check_global_placement(g);
     graphs[i] = std::move(g);
   };
-  parallel_for(N, lower_one);
+  parallel_for(N, lower_one, true);
   for (const NetGraph& g : graphs) {
     hp.max_checkpoint_segments = std::max(hp.max_checkpoint_segments, g.checkpoint_segments);
     hp.sum_global_elems += g.global_elems;

@@ -3,6 +3,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <complex>
 #include <cstdint>
 #include <exception>
@@ -62,24 +63,47 @@ qtc_status guarded(F&& f) {
 
 // Runs f(0) .. f(n - 1) on several host threads (fewer where the system refuses more).
 // Every call has ended on return; the exception of the lowest index is thrown again.
+// Starting a thread takes some 20 us, so unless the calls are known to be long (eager),
+// the caller begins alone and takes a helper per 200 us of work that its calls so far
+// let it expect.
 template <typename F>
-void parallel_for(int n, F&& f) {
+void parallel_for(int n, F&& f, bool eager = false) {
+  using Clock = std::chrono::steady_clock;
   std::vector<std::exception_ptr> errors(n);
   std::atomic<int> next{0};
-  auto work = [&]() noexcept {
-    for (int i = next++; i < n; i = next++) try {
-        f(i);
-      } catch (...) {
-        errors[i] = std::current_exception();
-      }
+  auto run = [&](int i) noexcept {
+    try {
+      f(i);
+    } catch (...) {
+      errors[i] = std::current_exception();
+    }
   };
-  const unsigned want = std::min({32u, std::thread::hardware_concurrency(), (unsigned)n});
+  auto work = [&]() noexcept {
+    for (int i = next++; i < n; i = next++) run(i);
+  };
   std::vector<std::thread> pool;
-  try {
-    pool.reserve(want);
-    for (unsigned t = 1; t < want; ++t) pool.emplace_back(work);
-  } catch (const std::exception&) {
-    // the threads there are do the work
+  auto grow = [&](double helpers) {
+    const double most = std::min({31.0, std::thread::hardware_concurrency() - 1.0, n - 1.0});
+    const int want = (int)std::max(0.0, std::min(helpers, most));
+    try {
+      pool.reserve(want);
+      for (int t = 0; t < want; ++t) pool.emplace_back(work);
+    } catch (const std::exception&) {
+      // the threads there are do the work
+    }
+  };
+  if (eager) {
+    grow(n - 1.0);
+  } else {
+    const auto start = Clock::now();
+    for (int i = next++; i < n; i = next++) {
+      run(i);
+      const double us = std::chrono::duration<double, std::micro>(Clock::now() - start).count();
+      const double helpers = us / (i + 1) * (n - 1 - i) / 200.0;
+      if (i < 8 && helpers < 2.0) continue;
+      grow(helpers);
+      break;
+    }
   }
   work();
   for (std::thread& th : pool) th.join();

@@ -253,7 +253,7 @@ void search_tree(const Plan& plan, bool alone, ExecutionTree& out) {
     totals[k] = walk(u, order);
   };
   if (alone) {
-    parallel_for(2, search);
+    parallel_for(2, search, true);
   } else {
     search(0);
     search(1);
