@@ -141,8 +141,8 @@ static_assert(sizeof(CLane) == 16, "one unit per lane");
 constexpr int kLaneDotSlots = 8;
 // Bytes of a graph-executor task's accumulators: FP64 in every element type, as its
 // slots are (a task sums all leaves of its subtree; in FP32 150 equal terms of 0.35 came
-// out 5e-7 off).  Dense p=2 n=100 value + gradient: 909 to 922 us, 900 with sums in
-// FP32; dots over several warps, with accumulators each, measured the same.
+// out 5e-7 off).  Dense p=2 n=100 value + gradient: 906 us, 900 with sums in FP32;
+// dots over several warps, with accumulators each, measured the same.
 QTC_HD inline uint32_t lane_dot_bytes(int n_params) { return 32u * 16u * (uint32_t)n_params; }
 constexpr uint32_t kSOpUnits = 5;
 // Units of half of a stage of `bytes` bytes (at most 8 KiB a half).

@@ -566,7 +566,7 @@ __device__ __forceinline__ void add_dot(double2& sum, float2 v, float2 d) {
 // lane are read before it, so a level of lanes costs about one round trip
 // through shared memory and the barrier (an op run from its record forms its
 // offsets first, 100 instructions or so).  The p=2 n=100 gradient launch (250
-// networks of about 485 ops in 163 levels): 209 -> 115 us.
+// networks of about 485 ops in 163 levels): 209 -> 105 us.
 template <typename T, int kLog, typename TeamT, typename At, typename A, typename G,
           typename Result>
 __device__ __forceinline__ void run_stream(const uint4* src, uint32_t batches, uint4* stage,

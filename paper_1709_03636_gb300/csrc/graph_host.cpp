@@ -595,7 +595,7 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
   // its lane accumulators of leaf dots and 1536 (else 512) for its stage, as long as
   // they cost no CTA per SM (other tasks stage more).  With 512 bytes, batches of 15
   // units, the whole-network tasks of dense p=2 n=100 took long enough for 1080 us in
-  // all (920 with 1536).
+  // all (906 with 1536).
   auto layout = [&](size_t beside) {
     hp.work_bytes =
         round16(std::max({beside + (size_t)max_arena * elem, chunk_task, tile_task}));
