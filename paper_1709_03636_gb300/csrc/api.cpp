@@ -1336,18 +1336,22 @@ static Prepared& prepare(qtc_engine* e, qtc_batch* b, int dtype, int want_grad,
       throw;
     }
   };
-  const HostProgram& hp = host_program(b, dtype, want_grad, max_dyn, e->options);
-  try {
-    return upload(hp);
-  } catch (const Error& err) {
-    // (warp programs have one form)
-    if (err.status != QTC_ERR_ARENA || hp.warp_teams) throw;
-  }
   // An arena that is too small for the faster form of the program: its smallest one
-  // (dense p=2 n=100: 4.6 MB of tables instead of 7.6, value + gradient 16.2 instead of 27.4).
-  ProgramOptions small = e->options;
-  small.compact = true;
-  return upload(host_program(b, dtype, want_grad, max_dyn, small));
+  // (dense p=2 n=100: 4.6 MB of tables instead of 7.4, value + gradient 16.2 instead of
+  // 27.4), and that along the plans' own trees, whose tensors may need less.
+  for (int form = 0;; ++form) {
+    ProgramOptions opts = e->options;
+    opts.compact = form >= 1;
+    opts.plan_trees = form >= 2;
+    const HostProgram& hp = host_program(b, dtype, want_grad, max_dyn, opts);
+    try {
+      return upload(hp);
+    } catch (const Error& err) {
+      // (warp programs have one form; trees differ in complex128 graph programs only)
+      const int forms = hp.graph ? (dtype == QTC_C128 ? 3 : 2) : hp.warp_teams ? 1 : 2;
+      if (err.status != QTC_ERR_ARENA || form + 1 == forms) throw;
+    }
+  }
 }
 
 static void launch(qtc_engine* e, const Prepared& pr, const double* params_dev, double* out_dev,

@@ -524,7 +524,7 @@ void build_graph_program(HostProgram& hp, const std::vector<Plan>& plans,
       graphs[i].units.push_back(std::move(u));
       return;
     }
-    const bool rearranged = hp.dtype == QTC_C128 && !opts.compact;
+    const bool rearranged = hp.dtype == QTC_C128 && !opts.plan_trees;
     NetGraph g = rearranged ? lower_network(i, execution_plan(plans[i], hp.dtype, N == 1))
                             : lower_network(i, plans[i]);
     if (rearranged && (!g.fits || over(g) || wide(g))) {

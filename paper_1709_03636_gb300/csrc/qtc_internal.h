@@ -378,15 +378,16 @@ struct ProgramOptions {
                                    // 2: per warp, steps always streamed
   int sm_count = 152;              // SMs of the device the program is laid out for
   bool graph_hi_occupancy = false; // graph executor: the five-CTAs-per-SM instantiation
-  bool compact = false;            // the smallest program tables: the plans' own trees, few lanes
-                                   // in the streams, no steps cut finer for few networks
+  bool compact = false;            // the smallest program tables: few lanes in the streams, no
+                                   // steps cut finer for few networks
+  bool plan_trees = false;         // graph executor: the plans' own trees in every element type
   bool operator==(const ProgramOptions& o) const {
     return wave_cap_bytes == o.wave_cap_bytes && force_graph == o.force_graph &&
            small_rank == o.small_rank && task_terms_log2 == o.task_terms_log2 &&
            tile_mode == o.tile_mode &&
            subtree_bytes == o.subtree_bytes && warp_teams == o.warp_teams &&
            sm_count == o.sm_count && graph_hi_occupancy == o.graph_hi_occupancy &&
-           compact == o.compact;
+           compact == o.compact && plan_trees == o.plan_trees;
   }
 };
 
